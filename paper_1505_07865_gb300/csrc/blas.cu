@@ -1,6 +1,7 @@
 // Vector kernels of the Krylov solvers (Sec. V: FGMRES outer, GMRES(N_s) inner).
 // Dot products use a fixed grid and a fixed-order final sum, so results are
 // bitwise reproducible run to run.
+#include <algorithm>
 #include <type_traits>
 
 #include "ibr_internal.cuh"
@@ -224,6 +225,45 @@ __global__ void __launch_bounds__(RED_THREADS) k_block_sums(long long m, int C, 
         block_sum_t<T, 1>(v, 1, o);
         if (threadIdx.x == 0) partial[(long long)blockIdx.x * C + c] = o[0];
     }
+}
+
+// The same with the rounding errors kept: each thread's sum is a pair (s, e), every
+// addition s + x split into its rounded value and its error by Knuth's two-sum
+// on the FP32 pipe (a plain FP64 accumulation would convert and add 8 M
+// entries at 1/64 of that rate); FP64 sums of the pairs.  FP64 x: plain sums.
+__device__ __forceinline__ void add_keep(float x, float& s, float& e) {
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+    s = t;
+}
+__device__ __forceinline__ void add_keep(double x, double& s, double&) { s += x; }
+
+// blockIdx.y: component c; partial[blk*C + c]; vec: m % 4 == 0 and x aligned for 4-entry loads
+template <typename T>
+__global__ void __launch_bounds__(RED_THREADS) k_block_sums_acc(long long m, int C, const T* __restrict__ x,
+                                                                double* __restrict__ partial, int vec) {
+    const int c = blockIdx.y;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    const T* xc = x + (long long)c * m;
+    T s0 = T(0), e0 = T(0), s1 = T(0), e1 = T(0);
+    if (vec) {
+        struct alignas(16) P4 {
+            T v[4];
+        };
+        for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < m / 4; q += stride) {
+            const P4 a = reinterpret_cast<const P4*>(xc)[q];
+            add_keep(a.v[0], s0, e0);
+            add_keep(a.v[1], s1, e1);
+            add_keep(a.v[2], s0, e0);
+            add_keep(a.v[3], s1, e1);
+        }
+    } else {
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += stride) add_keep(xc[i], s0, e0);
+    }
+    double v[1] = {((double)s0 + (double)s1) + ((double)e0 + (double)e1)};
+    __shared__ double o[1];
+    block_sum<1>(v, o);
+    if (threadIdx.x == 0) partial[(long long)blockIdx.x * C + c] = o[0];
 }
 
 __global__ void k_scale_vals(int C, double s, double* v) {
@@ -1569,6 +1609,17 @@ void block_means(long long m, int C, const T* x, double* partial, double* out, c
     IBR_CHECK_LAUNCH();
 }
 template <typename T>
+void block_means_acc(long long m, int C, const T* x, double* partial, double* out, cudaStream_t s) {
+    ProfScope ps(KID_BLOCK_MEANS, s, (double)m * C * sizeof(T));
+    const int blocks = (int)std::min<long long>(RED_BLOCKS / 4, (m / 4 + RED_THREADS - 1) / RED_THREADS + 1);
+    k_block_sums_acc<T><<<dim3(blocks, C), RED_THREADS, 0, s>>>(m, C, x, partial, m % 4 == 0 && vec16(x) ? 1 : 0);
+    IBR_CHECK_LAUNCH();
+    k_finalize<<<C, RED_THREADS, 0, s>>>(partial, blocks, C, out);
+    IBR_CHECK_LAUNCH();
+    k_scale_vals<<<1, 32, 0, s>>>(C, 1.0 / (double)m, out);
+    IBR_CHECK_LAUNCH();
+}
+template <typename T>
 void subtract_means(long long m, int C, T* x, const double* means, cudaStream_t s) {
     ProfScope ps(KID_SUB_MEANS, s, 2.0 * m * C * sizeof(T));
     if (m % 4 == 0 && vec16(x))
@@ -1605,6 +1656,7 @@ void hess_solve(const double* H, int ldh, const double* gv, int k, double* y, cu
                                   cudaStream_t);                                                                \
     template void norm2<T>(long long, const T*, double*, double*, cudaStream_t);                                \
     template void block_means<T>(long long, int, const T*, double*, double*, cudaStream_t);                     \
+    template void block_means_acc<T>(long long, int, const T*, double*, double*, cudaStream_t);                 \
     template void subtract_means<T>(long long, int, T*, const double*, cudaStream_t);
 IBR_INST(double)
 IBR_INST(float)

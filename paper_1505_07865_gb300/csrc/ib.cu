@@ -271,7 +271,8 @@ __global__ void k_spread_gather(long long F, const long long* __restrict__ face,
 // one warp per marker; lanes stride the KW^D support of each component
 template <int D, int KW, typename T, typename Tadd>
 __global__ void k_interp(Geo g, int N, const int* __restrict__ idx, const T* __restrict__ w, const T* __restrict__ v,
-                         T* __restrict__ out, T sign, const Tadd* __restrict__ add, T add_scale) {
+                         T* __restrict__ out, T sign, const Tadd* __restrict__ add, T add_scale,
+                         const double* __restrict__ mean) {
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (warp >= N) return;
@@ -300,7 +301,8 @@ __global__ void k_interp(Geo g, int N, const int* __restrict__ idx, const T* __r
         }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) {
-            T r = sign * acc;
+            // the weights of a window sum to one: J (v - m) = J v - m
+            T r = sign * (mean ? acc - (T)mean[a] : acc);
             if (add) r += add_scale * (T)add[ia];
             out[ia] = r;
         }
@@ -474,7 +476,7 @@ void spread_gather(const MarkerData& md, const T* lam, T* y, double scale, cudaS
 
 template <typename T, typename Tadd>
 void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign, const Tadd* add, cudaStream_t s,
-            double add_scale) {
+            double add_scale, const double* mean) {
     const T* w = sizeof(T) == 8 ? reinterpret_cast<const T*>(md.w64) : reinterpret_cast<const T*>(md.w32);
     int threads = 128;
     int blocks = grid_1d((long long)md.N * 32, threads);
@@ -483,14 +485,18 @@ void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign,
                  (double)md.N * g.d * ((g.d == 3 ? kw * kw * kw : kw * kw) * sizeof(T) + g.d * kw * sizeof(T) + sizeof(T)));
     if (g.d == 3) {
         if (kw == 6)
-            k_interp<3, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
+            k_interp<3, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
+                                                          mean);
         else
-            k_interp<3, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
+            k_interp<3, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
+                                                          mean);
     } else {
         if (kw == 6)
-            k_interp<2, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
+            k_interp<2, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
+                                                          mean);
         else
-            k_interp<2, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
+            k_interp<2, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
+                                                          mean);
     }
     IBR_CHECK_LAUNCH();
 }
@@ -518,9 +524,9 @@ void rigid_KT(int d, int B, const int* body_start, const double* rel, const doub
 template void spread_gather<double>(const MarkerData&, const double*, double*, double, cudaStream_t);
 template void spread_gather<float>(const MarkerData&, const float*, float*, double, cudaStream_t);
 template void interp<double, double>(const Geo&, const MarkerData&, const double*, double*, double, const double*,
-                                     cudaStream_t, double);
+                                     cudaStream_t, double, const double*);
 template void interp<float, double>(const Geo&, const MarkerData&, const float*, float*, double, const double*,
-                                    cudaStream_t, double);
+                                    cudaStream_t, double, const double*);
 template void lam_sum<double>(int, int, const double*, double, double*, cudaStream_t);
 template void lam_sum<float>(int, int, const float*, double, double*, cudaStream_t);
 

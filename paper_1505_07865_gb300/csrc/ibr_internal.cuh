@@ -367,6 +367,9 @@ void combine(long long n, const Tz* Z, long long ld, int k, const double* y, T* 
 // x_c -= mean_c for the blocks selected by mask
 template <typename T>
 void block_means(long long m, int C, const T* x, double* partial, double* out, cudaStream_t s);
+// the same with error-compensated partial sums (exact to FP64 rounding also for FP32 x)
+template <typename T>
+void block_means_acc(long long m, int C, const T* x, double* partial, double* out, cudaStream_t s);
 template <typename T>
 void subtract_means(long long m, int C, T* x, const double* means, cudaStream_t s);
 
@@ -461,10 +464,11 @@ void markers_build_gather(const Geo& g, MarkerData& md, cudaStream_t s);
 // y[face] += scale * sum w * lam   (no atomics; one thread per touched face)
 template <typename T>
 void spread_gather(const MarkerData& md, const T* lam, T* y, double scale, cudaStream_t s);
-// out[i*d+a] = sign * (J v)_i^a + (add ? add_scale * add[i*d+a] : 0)
+// out[i*d+a] = sign * (J (v - mean))_i^a + (add ? add_scale * add[i*d+a] : 0);
+// mean: d doubles on the device or NULL (zero)
 template <typename T, typename Tadd>
 void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign, const Tadd* add,
-            cudaStream_t s, double add_scale);
+            cudaStream_t s, double add_scale, const double* mean = nullptr);
 // shift[a] = scale * sum_i lam[i*d+a]  (double, a < d)
 template <typename T>
 void lam_sum(int d, int N, const T* lam, double scale, double* shift, cudaStream_t s);

@@ -202,6 +202,7 @@ struct ibr_grid {
     // bytes per entry); vk64: in the double-float case the FP64 copy of the
     // current basis vector that the preconditioner reads
     double *V = nullptr, *Z = nullptr, *b = nullptr, *x = nullptr, *w = nullptr, *vk64 = nullptr;
+    double* xc = nullptr;  // the iterate at the start of a cycle that goes on after its first residual
     double *H = nullptr, *cs = nullptr, *sn = nullptr, *gv = nullptr, *yv = nullptr;
     double *h1 = nullptr, *h2 = nullptr, *sc = nullptr, *partial = nullptr, *shift = nullptr, *means = nullptr;
     double *hk2 = nullptr, *st = nullptr;
@@ -461,14 +462,22 @@ struct PC {
                 inner_gmres(rs2, xs);
             }
         }
-        // keep the Krylov vectors in the space of the constrained problem:
-        // <v> = 0 (periodic steady Stokes) and <pi> = 0
-        block_means<T>(n, d + 1, xs, partial, means, s);
-        if (G->null_v())
-            subtract_means<T>(n, d + 1, xs, means, s);
-        else
-            subtract_means<T>(n, 1, xs + (long long)d * n, means + d, s);
+        // <v> = 0 (periodic steady Stokes) and <pi> = 0 are part of the
+        // constrained problem.  Uniform fields lie in the null space of the fluid
+        // rows, so the vector itself is left as it is and only the mean velocity
+        // is measured: the product with the matrix takes it out of the
+        // constraint rows (full_matvec), and the solution is projected at the
+        // end of each cycle.  Subtracting it from the entries in the
+        // preconditioner's precision left a mean of about 1e-9 |v| after
+        // rounding, which the final projection turned into an error of the
+        // constraints: 128^3 solves to 3e-10 stopped there and took a second
+        // cycle (43 iterations; 31 without it).
+        if (G->null_v() && N > 0) block_means_acc<T>(n, d, xs, partial, means, s);
     }
+
+    // the mean velocity of the last apply's result (d doubles on the device),
+    // NULL where the constraint rows do not need it
+    const double* mean_v() const { return G->null_v() && G->N > 0 ? means : nullptr; }
 
     static bool use_graphs() {
         static const bool off = [] {
@@ -581,7 +590,7 @@ void free_markers(ibr_grid* G) {
 
 void free_outer(ibr_grid* G) {
     double** ps[] = {&G->V, &G->Z, &G->b, &G->x, &G->w, &G->H, &G->cs, &G->sn, &G->gv, &G->yv,
-                     &G->h1, &G->h2, &G->sc, &G->partial, &G->shift, &G->means, &G->hk2, &G->st, &G->vk64};
+                     &G->h1, &G->h2, &G->sc, &G->partial, &G->shift, &G->means, &G->hk2, &G->st, &G->vk64, &G->xc};
     for (double** p : ps) dfree(*p);
     dfree(G->wait_err);
     G->m_alloc = 0;
@@ -1130,6 +1139,7 @@ void ensure_outer(ibr_grid* G, int m) {
     G->Z = dalloc<double>((size_t)m * len);
     G->b = dalloc<double>(len);
     G->x = dalloc<double>(len);
+    G->xc = dalloc<double>(len);
     G->w = dalloc<double>(lp);
     IBR_CUDA_TRY(cudaMemsetAsync(G->w, 0, lp * sizeof(double), G->stream));
     G->H = dalloc<double>((size_t)(m + 1) * (m + 1));
@@ -1152,8 +1162,10 @@ void ensure_outer(ibr_grid* G, int m) {
     G->m_alloc = m;
 }
 
-// y = (system matrix) x  (FP64)
-void full_matvec(ibr_grid* G, const double* x, double* y) {
+// y = (system matrix) x  (FP64); mean_v: the mean velocity of x (device, d
+// doubles), taken out of the velocity before it is interpolated (NULL: x has
+// mean zero, or is taken as it is)
+void full_matvec(ibr_grid* G, const double* x, double* y, const double* mean_v = nullptr) {
     cudaStream_t s = G->stream;
     const Geo& g = G->geo;
     int d = G->d;
@@ -1167,7 +1179,7 @@ void full_matvec(ibr_grid* G, const double* x, double* y) {
     stokes_apply<double>(g, x, y, G->sigma(), G->eta, shift, s);
     if (G->N > 0) {
         spread_gather<double>(G->md, lam, y, -1.0 / std::pow(g.h, d), s);
-        interp<double, double>(g, G->md, x, y + nS, -1.0, nullptr, s, 0.0);
+        interp<double, double>(g, G->md, x, y + nS, -1.0, nullptr, s, 0.0, mean_v);
     }
     if (G->nfree > 0) {
         // free bodies: -J v + K_f U_f on their markers, and K_f^T Lambda
@@ -1179,11 +1191,14 @@ void full_matvec(ibr_grid* G, const double* x, double* y) {
 }
 
 // fluid_prepared: the FP32 copy of r's fluid part is already in pc32->rs
-void pc_apply(ibr_grid* G, const double* r, double* z, bool fluid_prepared) {
-    if (G->precision == IBR_FP64)
+// returns the mean velocity of z (PC::mean_v)
+const double* pc_apply(ibr_grid* G, const double* r, double* z, bool fluid_prepared) {
+    if (G->precision == IBR_FP64) {
         G->pc64->apply(r, z);
-    else
-        G->pc32->apply(r, z, fluid_prepared);
+        return G->pc64->mean_v();
+    }
+    G->pc32->apply(r, z, fluid_prepared);
+    return G->pc32->mean_v();
 }
 
 double read_scalar(ibr_grid* G, const double* dev) {
@@ -1228,6 +1243,14 @@ int arnoldi_kind(long long len) {
 }
 
 // warm: start from the x already in G->x (time stepping), else from x = 0
+//
+// When the Givens estimate meets the target, the iterate is formed and its true
+// residual taken.  Where rounding has left that above the target, the cycle goes
+// on with the basis it has and a stricter estimate (the iterate at its start is
+// kept in xc), instead of being given up: a new cycle starts from a residual of
+// rounding noise and needs about ten steps to gain what one or two more steps of
+// the old one do.  Where going on does not help (the residual stays above three
+// quarters of what it was), the cycle ends there as it would have.
 int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm = false) {
     cudaStream_t s = G->stream;
     long long len = G->len;
@@ -1253,40 +1276,34 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
     bool last_cycle_converged_est = false;
     int stalls = 0;
     double last_rn = 0.0;
-    int status = IBR_OK;
-    while (true) {
-        // r = b - A x  (into w)
-        if (first) {
-            IBR_CUDA_TRY(cudaMemcpyAsync(G->w, G->b, len * sizeof(double), cudaMemcpyDeviceToDevice, s));
-        } else {
-            full_matvec(G, G->x, G->w);
-            vec_axpby<double>(len, 1.0, G->b, -1.0, G->w, s);
-        }
+    // w = b - A x and its norm
+    auto residual = [&] {
+        full_matvec(G, G->x, G->w);
+        vec_axpby<double>(len, 1.0, G->b, -1.0, G->w, s);
         norm2<double>(len, G->w, G->partial, G->sc + 0, s);
-        double rn = std::sqrt(read_scalar(G, G->sc + 0));
+        return std::sqrt(read_scalar(G, G->sc + 0));
+    };
+    // r = b - A x (into w)
+    double rn = bnorm;
+    if (first)
+        IBR_CUDA_TRY(cudaMemcpyAsync(G->w, G->b, len * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    else
+        rn = residual();
+    while (true) {
         info.rel_res_true = rn / bnorm;
         if (verbose) std::fprintf(stderr, "[ibr] restart %d true rel res %.3e\n", info.restarts, rn / bnorm);
         if (std::isnan(rn)) throw Error{IBR_ENUMERIC, "NaN in the FGMRES residual"};
-        if (rn <= target) break;
+        if (rn <= target) return IBR_OK;
         // a cycle that ended on the Givens estimate but left the true residual
         // where it was has hit the attainable accuracy of FP64 for this
         // scaling: stop after three such cycles instead of spinning
         if (!first && last_cycle_converged_est) {
             stalls = (rn > 0.5 * last_rn) ? stalls + 1 : 0;
-            if (stalls >= 3) {
-                status = IBR_ENOTCONV;
-                break;
-            }
+            if (stalls >= 3) return IBR_ENOTCONV;
         }
         last_rn = rn;
-        if (info.iters >= o.max_iters) {
-            status = IBR_ENOTCONV;
-            break;
-        }
-        if (o.time_cap_ms > 0 && now_ms() - t0 > o.time_cap_ms) {
-            status = IBR_ETIMEOUT;
-            break;
-        }
+        if (info.iters >= o.max_iters) return IBR_ENOTCONV;
+        if (o.time_cap_ms > 0 && now_ms() - t0 > o.time_cap_ms) return IBR_ETIMEOUT;
         givens_init(G->sc + 0, G->gv, m + 1, G->sc + 1, G->sc + 2, s);
         // V_0 = r / |r|; in mixed precision the preconditioner's FP32 copy of
         // its fluid part is written by the same pass
@@ -1306,13 +1323,13 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
         } else {
             scale_rsqrt<double, double>(lp, G->sc + 2, G->w, G->V, nullptr, 0, s);
         }
-        int k = 0;
+        double est_target = target, trial_rn = 0.0;
         last_cycle_converged_est = false;
         for (int j = 0; j < m; ++j) {
             double* Zj = G->Z + (long long)j * len;
             double* Vj = G->V + (long long)j * lp;
-            pc_apply(G, df ? G->vk64 : Vj, Zj, true);
-            full_matvec(G, Zj, G->w);
+            const double* mv = pc_apply(G, df ? G->vk64 : Vj, Zj, true);
+            full_matvec(G, Zj, G->w, mv);
             // the FP64 basis: the preconditioner reads V_{j+1} itself (and, mixed,
             // the FP32 copy of its fluid part in rs32)
             if (arn == ARN_MGS) {
@@ -1324,7 +1341,6 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
             }
             arnoldi_column(G->H, m + 1, G->h1, arn == ARN_MGS ? nullptr : G->h2, G->st + 2, j, G->cs, G->sn, G->gv,
                            G->sc + 3, G->sc + 4, s);
-            k = j + 1;
             info.iters++;
             double est = read_scalar(G, G->sc + 3);
             info.rel_res_est = est / bnorm;
@@ -1335,24 +1351,33 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
                              est / bnorm, hn, (int)re);
             }
             if (std::isnan(est)) throw Error{IBR_ENUMERIC, "NaN in the FGMRES Arnoldi process"};
+            const bool timeout = o.time_cap_ms > 0 && now_ms() - t0 > o.time_cap_ms;
+            const bool last = j + 1 == m || info.iters >= o.max_iters || timeout;
+            if (est > est_target && !last) continue;
             if (est <= target) last_cycle_converged_est = true;
-            if (est <= target || info.iters >= o.max_iters) break;
-            if (o.time_cap_ms > 0 && now_ms() - t0 > o.time_cap_ms) break;
+            {
+                // the pipelined Gram-Schmidt passes flag a wait that timed out
+                int werr = 0;
+                IBR_CUDA_TRY(cudaMemcpyAsync(&werr, G->wait_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+                IBR_CUDA_TRY(cudaStreamSynchronize(s));
+                if (werr) throw Error{IBR_ECUDA, "a pipelined Gram-Schmidt pass timed out waiting for its copies"};
+            }
+            if (trial_rn > 0.0)  // back to the iterate at the cycle's start
+                IBR_CUDA_TRY(cudaMemcpyAsync(G->x, G->xc, len * sizeof(double), cudaMemcpyDeviceToDevice, s));
+            else if (!last)
+                IBR_CUDA_TRY(cudaMemcpyAsync(G->xc, G->x, len * sizeof(double), cudaMemcpyDeviceToDevice, s));
+            hess_solve(G->H, m + 1, G->gv, j + 1, G->yv, s);
+            combine<double, double>(len, G->Z, len, j + 1, G->yv, G->x, true, s);
+            project_solution(G, G->x);
+            rn = residual();
+            if (rn <= target || last || !(est > 0.0) || !(rn < 1e3 * target)) break;
+            if (trial_rn > 0.0 && rn > 0.75 * trial_rn) break;
+            trial_rn = rn;
+            est_target = 0.5 * std::min(est, target) * (target / rn);
         }
-        {
-            // the pipelined Gram-Schmidt passes flag a wait that timed out
-            int werr = 0;
-            IBR_CUDA_TRY(cudaMemcpyAsync(&werr, G->wait_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-            IBR_CUDA_TRY(cudaStreamSynchronize(s));
-            if (werr) throw Error{IBR_ECUDA, "a pipelined Gram-Schmidt pass timed out waiting for its copies"};
-        }
-        hess_solve(G->H, m + 1, G->gv, k, G->yv, s);
-        combine<double, double>(len, G->Z, len, k, G->yv, G->x, true, s);
-        project_solution(G, G->x);
         info.restarts++;
         first = false;
     }
-    return status;
 }
 
 }  // namespace
@@ -1510,7 +1535,7 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
     const int m = restart;
     double t = 0.0;
     // outer FGMRES
-    t += pg(8.0 * (m + 1) * lp) + pg(8.0 * m * len) + 3 * pg(8.0 * len) + pg(8.0 * lp);
+    t += pg(8.0 * (m + 1) * lp) + pg(8.0 * m * len) + 4 * pg(8.0 * len) + pg(8.0 * lp);
     t += 8.0 * ((m + 1) * (m + 1) + 8 * (m + 2)) + pg(8.0 * RED_BLOCKS * std::max(m + 1, 4));
     // preconditioner: coarse multigrid levels (d stacked fields, u and f)
     Geo c = g;
