@@ -260,9 +260,6 @@ void mg_residual_restrict(const Geo& gf, const Geo& gc, const T* u, const T* f, 
                           double sigma, double kappa, cudaStream_t s);
 template <typename T>
 void mg_prolong_correct(const Geo& gf, const Geo& gc, T* u, const T* uc, int C, int fld0, cudaStream_t s);
-template <typename T>
-void mg_coarse_solve(const Geo& g, T* u, const T* f, int C, int fld0, double sigma, double kappa, int sweeps,
-                     cudaStream_t s);
 // One V-cycle for (sigma I - kappa Delta_h) U[0] = F0 on the levels lev[0..L)
 // (C stacked fields): red-black pre/post sweeps, averaging restriction into
 // Fw[l] (l >= 1), (bi/tri)linear prolongation, coarsest level by red-black
@@ -274,11 +271,15 @@ constexpr size_t MG_TAIL_MAX_SMEM = 200 * 1024;
 // rb_u, rb_f: scratch of C * lev[0].ncell each (or NULL): with them a periodic
 // 3-D finest level (n0 a multiple of 8) of a zero-start V-cycle with pre, post
 // >= 1 runs in red-black split layout (the same arithmetic, bitwise); rb_u1,
-// rb_f1 (C * lev[1].ncell each, or NULL) do the same for level 1
+// rb_f1 (C * lev[1].ncell each, or NULL) do the same for level 1.
+// Wt[l] (C * lev[l].ncell each, or NULL; Wt itself may be NULL): a temporary of
+// level l, with which it may run each of its legs in one launch
 template <typename T>
 void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, int C, int fld0, double sigma,
                double kappa, bool zero_start, int pre, int post, int coarse_sweeps, cudaStream_t s,
-               T* rb_u = nullptr, T* rb_f = nullptr, T* rb_u1 = nullptr, T* rb_f1 = nullptr);
+               T* rb_u = nullptr, T* rb_f = nullptr, T* rb_u1 = nullptr, T* rb_f1 = nullptr, T* const* Wt = nullptr);
+// levels that may run each leg in one launch (and need a temporary for it)
+inline bool mg_leg_level(const Geo& g) { return g.d == 2; }
 // red-black sweeps of the coarsest-level solve: enough for a preconditioner
 // (the coarsest grid has at most a few hundred cells)
 inline int mg_coarse_sweeps(const Geo& g) {

@@ -67,6 +67,7 @@ template <typename T>
 struct Multigrid {
     std::vector<Geo> lev;
     std::vector<T*> u, f;  // index 0 unused (caller's buffers)
+    std::vector<T*> tmp;   // per level: the temporary of its one-launch legs (NULL: none)
     T *rb_u = nullptr, *rb_f = nullptr;    // finest level in red-black split layout (periodic 3-D)
     T *rb_u1 = nullptr, *rb_f1 = nullptr;  // level 1 in the same layout
     int cmax = 0;
@@ -99,6 +100,7 @@ struct Multigrid {
             g = c;
         }
         coarse_sweeps = mg_coarse_sweeps(lev.back());
+        for (const Geo& l : lev) tmp.push_back(mg_leg_level(l) ? dalloc<T>((size_t)cmax * l.ncell) : nullptr);
         if (g0.d == 3 && !g0.wall && g0.n0 % 8 == 0 && lev.size() > 1) {
             rb_u = dalloc<T>((size_t)cmax * g0.ncell);
             rb_f = dalloc<T>((size_t)cmax * g0.ncell);
@@ -115,6 +117,8 @@ struct Multigrid {
         dfree(rb_f1);
         for (auto& p : u) dfree(p);
         for (auto& p : f) dfree(p);
+        for (auto& p : tmp) dfree(p);
+        tmp.clear();
         u.clear();
         f.clear();
         lev.clear();
@@ -127,7 +131,7 @@ struct Multigrid {
         std::vector<T*> U(u);
         U[0] = u0;
         mg_vcycle<T>(lev.data(), L, U.data(), f.data(), f0, C, fld0, sigma, kappa, zero_start, pre, post,
-                     coarse_sweeps, s, rb_u, rb_f, rb_u1, rb_f1);
+                     coarse_sweeps, s, rb_u, rb_f, rb_u1, rb_f1, tmp.data());
     }
 };
 
@@ -1370,10 +1374,10 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
             combine<double, double>(len, G->Z, len, j + 1, G->yv, G->x, true, s);
             project_solution(G, G->x);
             rn = residual();
-            if (rn <= target || last || !(est > 0.0) || !(rn < 1e3 * target)) break;
-            if (trial_rn > 0.0 && rn > 0.75 * trial_rn) break;
+            const double noise2 = rn * rn - est * est;
+            if (rn <= target || last || !(noise2 < target * target)) break;
             trial_rn = rn;
-            est_target = 0.5 * std::min(est, target) * (target / rn);
+            est_target = 0.7 * std::sqrt(target * target - std::max(noise2, 0.0));
         }
         info.restarts++;
         first = false;
@@ -1548,6 +1552,16 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
     }
     t += pg(e * (ns + 1) * nS) + pg(e * ns * nS) + 4 * pg(e * nS) + pg(e * d * nc) + 3 * pg(e * nc);
     t += pg(8.0 * RED_BLOCKS * std::max(ns + 1, 4)) + 2 * pg(e * dN) + pg(8.0 * dN);
+    // the temporaries of the one-launch legs (2-D)
+    Geo lg = g;
+    for (;;) {
+        if (mg_leg_level(lg)) t += pg(e * d * (double)lg.ncell);
+        if (!Multigrid<float>::can_coarsen(lg)) break;
+        lg.n0 /= 2;
+        lg.n1 /= 2;
+        if (d == 3) lg.n2 /= 2;
+        lg.ncell = (long long)lg.n0 * lg.n1 * lg.n2;
+    }
     // the red-black split copies of u and f of the finest level and level 1 (periodic 3-D)
     if (d == 3 && g.n0 % 8 == 0) t += 2 * pg(e * d * nc);
     if (d == 3 && g.n0 % 16 == 0 && Multigrid<float>::can_coarsen(g)) t += 2 * pg(e * d * nc / 8);
@@ -1573,6 +1587,7 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
             c2.ncell = (long long)c2.n0 * c2.n1 * c2.n2;
             mg64 += 2 * pg(8.0 * d * (double)c2.ncell);
         }
+        if (mg_leg_level(g)) mg64 += 4.0 / 3.0 * 8.0 * d * nc + 8 * pg(2097152.0);
         t += mg64 + pg(8.0 * (PAIR_NS + 1) * nS) + pg(8.0 * PAIR_NS * nS) + 8 * pg(8.0 * nS) + pg(8.0 * d * nc) +
              3 * pg(8.0 * nc);
         if (dN <= (double)pair_full_max()) blk2 = blkmax = dN * dN;

@@ -289,8 +289,8 @@ __global__ void __launch_bounds__(256) k_stokes_fx(const double* __restrict__ x,
     y[D * g.ncell + n.c] = val;
 }
 
-// ---- point operators shared by the per-level kernels and the one-CTA tail ----
-// (same arithmetic, so a level gives the same result on either path)
+// ---- point operators of the per-level kernels (the legs, the tail and the cluster
+// kernel apply the same formulas to cells in shared memory) ----
 
 // inv_diag = 1 / (sigma + 2D kh2), formed by rbgs_inv_diag on host or device
 template <int D, typename T>
@@ -317,19 +317,6 @@ __device__ __forceinline__ void rbgs_cell(T* u, const T* f, const Geo& g, int fl
         T dinv = wi.adj == 0 ? inv_diag : T(1) / (sigma + kh2 * T(2 * D - wi.adj));
         u[n.c] = (f[n.c] + kh2 * nb) * dinv;
     }
-}
-
-// the same for the t-th cell of the given colour (x index ih = t mod n0/2);
-// dh, d1: division by n0/2 and by n1
-template <int D, bool W, typename T>
-__device__ __forceinline__ void rbgs_point(T* u, const T* f, const Geo& g, int fld, T sigma, T kh2, T inv_diag,
-                                           int color, int zero_init, int t, FastDiv dh, FastDiv d1) {
-    const int hn0 = g.n0 >> 1;
-    const int r = fdiv(t, dh);
-    const int ih = t - r * hn0;
-    const int k = fdiv(r, d1);
-    const int j = r - k * g.n1;
-    rbgs_cell<D, W, T>(u, f, g, fld, sigma, kh2, inv_diag, zero_init, 2 * ih + ((j + k + color) & 1), j, k);
 }
 
 // residual f - (sigma u - kh2 Lap u) at fine cell (i, j, k)
@@ -395,16 +382,6 @@ __device__ __forceinline__ T restrict_cell(const T* u, const T* f, const Geo& gf
                 acc += fw[0][p] * fw[1][q] * fw[2][r] *
                        resid_cell<D, true, T>(u, f, gf, fld, sigma, kh2, fi[0][p], fi[1][q], fi[2][r]);
     return acc;
-}
-
-template <int D, bool W, typename T>
-__device__ __forceinline__ T restrict_point(const T* u, const T* f, const Geo& gf, const Geo& gc, int fld, T sigma,
-                                            T kh2, int t, FastDiv dc0, FastDiv dc1) {
-    const int r = fdiv(t, dc0);
-    const int I = t - r * gc.n0;
-    const int K = fdiv(r, dc1);
-    const int J = r - K * gc.n1;
-    return restrict_cell<D, W, T>(u, f, gf, fld, sigma, kh2, I, J, K);
 }
 
 // fine cell (i, j, k): cell-centred (bi/tri)linear interpolation of the coarse
@@ -492,70 +469,6 @@ __device__ __forceinline__ T prolong_cell(const T* cc, const Geo& gc, int fld, i
     return acc;
 }
 
-template <int D, bool W, typename T>
-__device__ __forceinline__ T prolong_point(const T* cc, const Geo& gf, const Geo& gc, int fld, int t, FastDiv df0,
-                                           FastDiv df1) {
-    const int r = fdiv(t, df0);
-    const int i = t - r * gf.n0;
-    const int k = fdiv(r, df1);
-    const int j = r - k * gf.n1;
-    return prolong_cell<D, W, T>(cc, gc, fld, i, j, k);
-}
-
-// block-wide mean of a[0..n) (all threads get it); red: 32 doubles of shared memory
-template <typename T>
-__device__ double block_mean(const T* a, int n, double* red) {
-    int tid = threadIdx.x, nt = blockDim.x;
-    double part = 0.0;
-    for (int c = tid; c < n; c += nt) part += (double)a[c];
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    __syncthreads();
-    if ((tid & 31) == 0) red[tid >> 5] = part;
-    __syncthreads();
-    if (tid < 32) {
-        double v = tid < (nt >> 5) ? red[tid] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (tid == 0) red[0] = v;
-    }
-    __syncthreads();
-    double m = red[0] / (double)n;
-    __syncthreads();
-    return m;
-}
-
-// coarsest-level solve in shared memory: for a singular field f (in sf,
-// modified) is made mean-free, u (su) from zero by red-black sweeps, then made
-// mean-free; d0, d1: division by n0 and n1
-template <int D, bool W, typename T>
-__device__ void coarse_block(T* su, T* sf, const Geo& g, int fld, T sigma, T kh2, T inv, int sweeps, double* red,
-                             FastDiv d0, FastDiv d1) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int nc = (int)g.ncell;
-    const bool sing = singular_field(g, fld, (double)sigma);
-    T fmean = sing ? (T)block_mean(sf, nc, red) : T(0);
-    for (int c = tid; c < nc; c += nt) {
-        sf[c] -= fmean;
-        su[c] = T(0);
-    }
-    __syncthreads();
-    for (int s = 0; s < sweeps; ++s) {
-        for (int color = 0; color < 2; ++color) {
-            for (int c = tid; c < nc; c += nt) {
-                const int r = fdiv(c, d0);
-                const int i = c - r * g.n0;
-                const int k = fdiv(r, d1);
-                const int j = r - k * g.n1;
-                if (((i + j + k) & 1) != color) continue;
-                rbgs_cell<D, W, T>(su, sf, g, fld, sigma, kh2, inv, 0, i, j, k);
-            }
-            __syncthreads();
-        }
-    }
-    T umean = sing ? (T)block_mean(su, nc, red) : T(0);
-    for (int c = tid; c < nc; c += nt) su[c] -= umean;
-    __syncthreads();
-}
-
 // red-black Gauss-Seidel half sweep on C stacked fields (component from blockIdx.z)
 template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_rbgs(T* __restrict__ u, const T* __restrict__ f, Geo g, int fld0, T sigma,
@@ -631,23 +544,6 @@ __global__ void __launch_bounds__(256) k_prolong(T* __restrict__ u, const T* __r
     u[cmp * gf.ncell + t] += prolong_cell<D, W, T>(uc + cmp * gc.ncell, gc, field_of(fld0, cmp), i, j, k);
 }
 
-// single-CTA coarse solve of the coarsest level (one CTA per field)
-template <int D, bool W, typename T>
-__global__ void __launch_bounds__(1024) k_coarse(T* __restrict__ u, const T* __restrict__ f, Geo g, int fld0,
-                                                 T sigma, T kh2, T inv, int sweeps, FastDiv d0, FastDiv d1) {
-    extern __shared__ unsigned char smem_raw[];
-    T* su = reinterpret_cast<T*>(smem_raw);
-    T* sf = su + g.ncell;
-    __shared__ double red[32];
-    int cmp = blockIdx.x;
-    const T* ff = f + cmp * g.ncell;
-    T* uu = u + cmp * g.ncell;
-    for (int c = threadIdx.x; c < (int)g.ncell; c += blockDim.x) sf[c] = ff[c];
-    __syncthreads();
-    coarse_block<D, W, T>(su, sf, g, field_of(fld0, cmp), sigma, kh2, inv, sweeps, red, d0, d1);
-    for (int c = threadIdx.x; c < (int)g.ncell; c += blockDim.x) uu[c] = su[c];
-}
-
 // The small levels of a V-cycle, all in one CTA's shared memory (one CTA per
 // field): levels tl.g[0] (finest of the tail) .. tl.g[nl-1] (coarsest), the
 // same sweeps, restriction, coarse solve and prolongation as the per-level
@@ -656,8 +552,9 @@ __global__ void __launch_bounds__(1024) k_coarse(T* __restrict__ u, const T* __r
 struct TailLevels {
     int nl;
     Geo g[MG_TAIL_MAX_LEVELS];
-    int uoff[MG_TAIL_MAX_LEVELS];
-    int foff[MG_TAIL_MAX_LEVELS];
+    int uoff[MG_TAIL_MAX_LEVELS];  // u, one array per colour
+    int foff[MG_TAIL_MAX_LEVELS];  // f, natural layout
+    int noff[MG_TAIL_MAX_LEVELS];  // the residual, then the level's result, natural layout
     FastDiv dh[MG_TAIL_MAX_LEVELS];  // n0 / 2
     FastDiv d0[MG_TAIL_MAX_LEVELS];  // n0
     FastDiv d1[MG_TAIL_MAX_LEVELS];  // n1
@@ -677,77 +574,356 @@ __device__ __forceinline__ T lev_inv(const L& tl, int l) {
     if constexpr (sizeof(T) == 4) return tl.invf[l]; else return tl.invd[l];
 }
 
-// the V-cycle over the levels of tl, whose finest level's f (and u unless
-// zero_start) are already in shared memory at sm; leaves u of the finest
-// level there.  Every thread of the CTA calls it.
+// coarse cell (I, J, K) of a wall grid from the fine residual r (natural layout):
+// restrict_cell's weights
+template <int D, typename T>
+__device__ __forceinline__ T tail_restrict_w(const T* r, const Geo& gf, int fld, int I, int J, int K) {
+    const int X[3] = {I, J, K};
+    int lo[3], cnt[3];
+    bool nrm[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        nrm[a] = a < D && ((gf.wall >> a) & 1) && fld == a;
+        if (nrm[a] && X[a] == 0) return T(0);
+        lo[a] = a >= D ? 0 : (nrm[a] ? 2 * X[a] - 1 : 2 * X[a]);
+        cnt[a] = a >= D ? 1 : (nrm[a] ? 3 : 2);
+    }
+    T acc = T(0);
+    for (int p = 0; p < cnt[0]; ++p)
+        for (int q = 0; q < cnt[1]; ++q)
+            for (int s = 0; s < cnt[2]; ++s) {
+                T w = nrm[0] ? (p == 1 ? T(0.5) : T(0.25)) : T(0.5);
+                w *= nrm[1] ? (q == 1 ? T(0.5) : T(0.25)) : T(0.5);
+                if (D == 3) w *= nrm[2] ? (s == 1 ? T(0.5) : T(0.25)) : T(0.5);
+                acc += w * r[lo[0] + p + gf.n0 * (lo[1] + q + gf.n1 * (lo[2] + s))];
+            }
+    return acc;
+}
+
+// A pair of cells of a level in shared memory: x = 2 ih and 2 ih + 1 of one row,
+// one cell of each colour, owned by one thread through the level's sweeps.  u is
+// kept as one array per colour, entry t = ih + (n0/2) row for the cell of that
+// colour in pair t: the neighbours of a colour's cell lie in the other colour's
+// array at entries t (the pair's other cell), t -+ 1 in the row, and t of the
+// adjacent rows and planes, so a warp reads consecutive words.
+template <int D>
+struct TailPair {
+    int t;                      // entry; the natural index of the pair's even cell is 2 t
+    int i, j, k;                // i = 2 ih
+    int xl, xr, ym, yp, zm, zp; // entries of the wrapped neighbours
+    int b;                      // colour of the even cell (the odd one's is 1 - b)
+};
+
+template <int D>
+__device__ __forceinline__ TailPair<D> tail_pair(const TailLevels& tl, int l, int t) {
+    const Geo& g = tl.g[l];
+    const int hn = g.n0 >> 1;
+    TailPair<D> p;
+    const int r = fdiv(t, tl.dh[l]);
+    const int ih = t - r * hn;
+    p.t = t;
+    p.k = D == 3 ? fdiv(r, tl.d1[l]) : 0;
+    p.j = r - p.k * g.n1;
+    p.i = 2 * ih;
+    p.xl = ih == 0 ? t + hn - 1 : t - 1;
+    p.xr = ih == hn - 1 ? t - hn + 1 : t + 1;
+    p.ym = p.j == 0 ? t + hn * (g.n1 - 1) : t - hn;
+    p.yp = p.j == g.n1 - 1 ? t - hn * (g.n1 - 1) : t + hn;
+    if (D == 3) {
+        const int pl = hn * g.n1;
+        p.zm = p.k == 0 ? t + pl * (g.n2 - 1) : t - pl;
+        p.zp = p.k == g.n2 - 1 ? t - pl * (g.n2 - 1) : t + pl;
+    } else {
+        p.zm = p.zp = 0;
+    }
+    p.b = (p.j + p.k) & 1;
+    return p;
+}
+
+// neighbour sum of the pair's cell of one colour: other = the other colour's
+// array, own = the pair's other cell, odd: this cell is the pair's odd one
+template <int D, bool W, typename T>
+__device__ __forceinline__ T tail_nbr(const TailPair<D>& p, const T* other, T own, bool odd, unsigned ok) {
+    if (!W) {
+        const T ex = other[odd ? p.xr : p.xl];
+        T s = own + ex + other[p.yp] + other[p.ym];
+        if (D == 3) s += other[p.zp] + other[p.zm];
+        return s;
+    }
+    T s = T(0);
+    if (ok & 1u) s += odd ? own : other[p.xl];
+    if (ok & 2u) s += odd ? other[p.xr] : own;
+    if (ok & 4u) s += other[p.ym];
+    if (ok & 8u) s += other[p.yp];
+    if (D == 3) {
+        if (ok & 16u) s += other[p.zm];
+        if (ok & 32u) s += other[p.zp];
+    }
+    return s;
+}
+
+// The V-cycle over the levels of tl, whose finest level's f (natural layout, at
+// foff) and, unless zero_start, u (one array per colour, at uoff) are already in
+// shared memory at sm; leaves u of the finest level in natural layout at noff.
+// Every thread of the block calls it.  The kernel runs on one SM, and the sweeps
+// issue few instructions per cell: each thread works out the places and keeps f
+// and u of its pairs (at most TAIL_NP of a level's) in registers once per
+// smoothing, and a half sweep is five loads, the update and a store per cell.
+// A level's sweeps are run by as many warps as it has pairs for, with a barrier
+// of their own; the other warps wait at the finer level's.  The tail of a 16^3
+// level took about 30 us with the places worked out in every half sweep.
+constexpr int TAIL_NP = 2;
+
 template <int D, bool W, typename T>
 __device__ void tail_solve(const TailLevels& tl, T* sm, int fld, T sigma, int zero_start, int pre, int post,
                            int sweeps, double* red) {
     const int tid = threadIdx.x, nt = blockDim.x;
-    auto half = [&](int l, int color, int zero) {
-        const Geo& g = tl.g[l];
-        const T kh2 = lev_kh2<T>(tl, l);
-        const T inv = lev_inv<T>(tl, l);
-        T* u = sm + tl.uoff[l];
-        const T* f = sm + tl.foff[l];
-        const int np = (int)(g.ncell >> 1);
-        for (int t = tid; t < np; t += nt)
-            rbgs_point<D, W, T>(u, f, g, fld, sigma, kh2, inv, color, zero, t, tl.dh[l], tl.d1[l]);
-        __syncthreads();
-    };
     const int L = tl.nl;
-    if (L == 1) {
-        const Geo& g = tl.g[0];
-        if (zero_start) {
-            coarse_block<D, W, T>(sm + tl.uoff[0], sm + tl.foff[0], g, fld, sigma, lev_kh2<T>(tl, 0),
-                                  lev_inv<T>(tl, 0), sweeps, red, tl.d0[0], tl.d1[0]);
-        } else {
-            for (int s = 0; s < sweeps; ++s) {
-                half(0, 0, 0);
-                half(0, 1, 0);
+    auto active = [&](int l) { return min(nt, ((int)(tl.g[l].ncell >> 1) + 31) & ~31); };
+    auto barrier = [&](int l) { asm volatile("bar.sync %0, %1;" ::"r"(1 + l), "r"(active(l)) : "memory"); };
+    // one level's share of this thread
+    TailPair<D> P[TAIL_NP];
+    T fv[TAIL_NP][2], v[TAIL_NP][2];  // by x: the pair's even and odd cell
+    T dinv[TAIL_NP][2];
+    unsigned ok[TAIL_NP][2];
+    int adj[TAIL_NP][2];
+    bool have[TAIL_NP];
+    auto open = [&](int l) {
+        const Geo& g = tl.g[l];
+        const int np = (int)(g.ncell >> 1), na = active(l);
+        const T* F = sm + tl.foff[l];
+        const T inv = lev_inv<T>(tl, l);
+#pragma unroll
+        for (int q = 0; q < TAIL_NP; ++q) {
+            const int t = tid + q * na;
+            have[q] = t < np && (q == 0 || na == nt);
+            if (!have[q]) continue;
+            P[q] = tail_pair<D>(tl, l, t);
+            fv[q][0] = F[2 * t];
+            fv[q][1] = F[2 * t + 1];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                ok[q][e] = 0x3Fu;
+                dinv[q][e] = inv;
+                if (W) {
+                    const WInfo wi = wall_info<D>(g, fld, P[q].i + e, P[q].j, P[q].k);
+                    ok[q][e] = wi.ident ? 0u : wi.ok;
+                    adj[q][e] = wi.ident ? 2 * D : wi.adj;  // a wall face: u = f, residual f - u
+                    if (wi.ident)
+                        dinv[q][e] = T(1);
+                    else if (wi.adj != 0)
+                        dinv[q][e] = T(1) / (sigma + lev_kh2<T>(tl, l) * T(2 * D - wi.adj));
+                }
             }
         }
-        return;
-    }
-    for (int l = 0; l + 1 < L; ++l) {
-        int zs = (l > 0) || zero_start;
-        if (pre == 0 && zs) {
-            T* u = sm + tl.uoff[l];
-            for (int c = tid; c < (int)tl.g[l].ncell; c += nt) u[c] = T(0);
-            __syncthreads();
-        }
-        for (int it = 0; it < pre; ++it) {
-            half(l, 0, zs && it == 0);
-            half(l, 1, 0);
-        }
-        const Geo& gf = tl.g[l];
-        const Geo& gc = tl.g[l + 1];
+    };
+    auto half = [&](int l, int color, bool zero) {
         const T kh2 = lev_kh2<T>(tl, l);
+        const int np = (int)(tl.g[l].ncell >> 1);
+        T* uc = sm + tl.uoff[l] + color * np;
+        const T* uo = sm + tl.uoff[l] + (1 - color) * np;
+#pragma unroll
+        for (int q = 0; q < TAIL_NP; ++q) {
+            if (!have[q]) continue;
+            const bool odd = P[q].b != color;
+            const int e = odd ? 1 : 0;
+            const T own = odd ? v[q][0] : v[q][1];
+            const T nb = zero ? T(0) : tail_nbr<D, W, T>(P[q], uo, own, odd, odd ? ok[q][1] : ok[q][0]);
+            const T un = ((odd ? fv[q][1] : fv[q][0]) + kh2 * nb) * (odd ? dinv[q][1] : dinv[q][0]);
+            if (e)
+                v[q][1] = un;
+            else
+                v[q][0] = un;
+            uc[P[q].t] = un;
+        }
+        barrier(l);
+    };
+    auto load_u = [&](int l) {
+        const int np = (int)(tl.g[l].ncell >> 1);
         const T* u = sm + tl.uoff[l];
-        const T* f = sm + tl.foff[l];
-        T* fc = sm + tl.foff[l + 1];
-        for (int t = tid; t < (int)gc.ncell; t += nt)
-            fc[t] = restrict_point<D, W, T>(u, f, gf, gc, fld, sigma, kh2, t, tl.d0[l + 1], tl.d1[l + 1]);
-        __syncthreads();
-    }
-    {
-        const Geo& g = tl.g[L - 1];
-        coarse_block<D, W, T>(sm + tl.uoff[L - 1], sm + tl.foff[L - 1], g, fld, sigma, lev_kh2<T>(tl, L - 1),
-                              lev_inv<T>(tl, L - 1), sweeps, red, tl.d0[L - 1], tl.d1[L - 1]);
-    }
-    for (int l = L - 2; l >= 0; --l) {
-        const Geo& gf = tl.g[l];
-        const Geo& gc = tl.g[l + 1];
-        T* u = sm + tl.uoff[l];
-        const T* uc = sm + tl.uoff[l + 1];
-        for (int t = tid; t < (int)gf.ncell; t += nt)
-            u[t] += prolong_point<D, W, T>(uc, gf, gc, fld, t, tl.d0[l], tl.d1[l]);
-        __syncthreads();
-        for (int it = 0; it < post; ++it) {
-            half(l, 1, 0);
-            half(l, 0, 0);
+#pragma unroll
+        for (int q = 0; q < TAIL_NP; ++q) {
+            if (!have[q]) continue;
+            v[q][0] = u[P[q].b * np + P[q].t];
+            v[q][1] = u[(1 - P[q].b) * np + P[q].t];
+        }
+    };
+    auto store_nat = [&](int l, T shift) {
+        T* N = sm + tl.noff[l];
+#pragma unroll
+        for (int q = 0; q < TAIL_NP; ++q) {
+            if (!have[q]) continue;
+            N[2 * P[q].t] = v[q][0] - shift;
+            N[2 * P[q].t + 1] = v[q][1] - shift;
+        }
+    };
+    // mean over the level's cells of this thread's values w (all its threads get it)
+    auto mean = [&](int l, T (&w)[TAIL_NP][2]) -> T {
+        const int na = active(l);
+        double part = 0.0;
+#pragma unroll
+        for (int q = 0; q < TAIL_NP; ++q)
+            if (have[q]) part += (double)w[q][0] + (double)w[q][1];
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (na > 32) {
+            barrier(l);
+            if ((tid & 31) == 0) red[tid >> 5] = part;
+            barrier(l);
+            part = 0.0;
+            for (int w2 = 0; w2 < (na >> 5); ++w2) part += red[w2];
+        }
+        return (T)(part / (double)tl.g[l].ncell);
+    };
+    // the coarsest level: for a singular field f is made mean-free, u from zero by
+    // red-black sweeps, then made mean-free
+    auto coarsest = [&](int l) {
+        const bool sing = singular_field(tl.g[l], fld, (double)sigma);
+        if (sing) {
+            const T m = mean(l, fv);
+#pragma unroll
+            for (int q = 0; q < TAIL_NP; ++q) {
+                fv[q][0] -= m;
+                fv[q][1] -= m;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < TAIL_NP; ++q) v[q][0] = v[q][1] = T(0);
+        for (int s = 0; s < sweeps; ++s) {
+            half(l, 0, s == 0);
+            half(l, 1, false);
+        }
+        store_nat(l, sing ? mean(l, v) : T(0));
+    };
+    if (tid < active(0)) {
+        if (L == 1) {
+            open(0);
+            if (zero_start) {
+                coarsest(0);
+            } else {
+                load_u(0);
+                for (int s = 0; s < sweeps; ++s) {
+                    half(0, 0, false);
+                    half(0, 1, false);
+                }
+                store_nat(0, T(0));
+            }
+        }
+        // down: sweeps, residual, restriction
+        int l = 0;
+        for (; l + 1 < L; ++l) {
+            const Geo& g = tl.g[l];
+            const bool zs = l > 0 || zero_start;
+            const T kh2 = lev_kh2<T>(tl, l);
+            const int np = (int)(g.ncell >> 1);
+            open(l);
+            if (!zs) {
+                load_u(l);
+            } else {
+#pragma unroll
+                for (int q = 0; q < TAIL_NP; ++q) v[q][0] = v[q][1] = T(0);
+                if (pre == 0) {
+#pragma unroll
+                    for (int q = 0; q < TAIL_NP; ++q)
+                        if (have[q]) sm[tl.uoff[l] + P[q].t] = sm[tl.uoff[l] + np + P[q].t] = T(0);
+                    barrier(l);
+                }
+            }
+            for (int it = 0; it < pre; ++it) {
+                half(l, 0, zs && it == 0);
+                half(l, 1, false);
+            }
+            T* R = sm + tl.noff[l];
+#pragma unroll
+            for (int q = 0; q < TAIL_NP; ++q) {
+                if (!have[q]) continue;
+                T res[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int col = e ? 1 - P[q].b : P[q].b;
+                    const T* uo = sm + tl.uoff[l] + (1 - col) * np;
+                    const T nb = tail_nbr<D, W, T>(P[q], uo, v[q][1 - e], e == 1, ok[q][e]);
+                    if (W && ok[q][e] == 0u)
+                        res[e] = fv[q][e] - v[q][e];
+                    else
+                        res[e] = fv[q][e] - (sigma * v[q][e] - kh2 * (nb + T((W ? adj[q][e] : 0) - 2 * D) * v[q][e]));
+                }
+                if (W) {
+                    R[2 * P[q].t] = res[0];
+                    R[2 * P[q].t + 1] = res[1];
+                } else {
+                    R[P[q].t] = res[0] + res[1];  // the two children in x of one coarse cell
+                }
+            }
+            barrier(l);
+            if (tid >= active(l + 1)) break;
+            const Geo& gc = tl.g[l + 1];
+            const int npc = (int)(gc.ncell >> 1), nac = active(l + 1);
+            T* Fc = sm + tl.foff[l + 1];
+#pragma unroll
+            for (int q = 0; q < TAIL_NP; ++q) {
+                const int t = tid + q * nac;
+                if (!(t < npc && (q == 0 || nac == nt))) continue;
+                const TailPair<D> pc = tail_pair<D>(tl, l + 1, t);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int I = pc.i + e;
+                    T acc = T(0);
+                    if (!W) {
+#pragma unroll
+                        for (int c = 0; c < (1 << (D - 1)); ++c) {
+                            const int dy = c & 1, dz = D == 3 ? (c >> 1) & 1 : 0;
+                            acc += R[I + gc.n0 * (2 * pc.j + dy + g.n1 * (2 * pc.k + dz))];
+                        }
+                        acc *= T(1) / T(1 << D);
+                    } else {
+                        acc = tail_restrict_w<D, T>(R, g, fld, I, pc.j, pc.k);
+                    }
+                    Fc[2 * t + e] = acc;
+                }
+            }
+        }
+        if (L > 1) {
+            if (l + 1 == L) {  // this thread has a share of the coarsest level
+                open(l);
+                coarsest(l);
+                --l;
+            }
+            // up from level l: the coarser levels' threads arrive when their result is stored
+            for (; l >= 0; --l) {
+                const Geo& g = tl.g[l];
+                const Geo& gc = tl.g[l + 1];
+                const int np = (int)(g.ncell >> 1);
+                barrier(l);
+                open(l);
+                load_u(l);
+                const T* Nc = sm + tl.noff[l + 1];
+#pragma unroll
+                for (int q = 0; q < TAIL_NP; ++q) {
+                    if (!have[q]) continue;
+#pragma unroll
+                    for (int col = 0; col < 2; ++col) {
+                        // the first half sweep overwrites colour 1 without reading it
+                        if (col == 1 && post > 0) continue;
+                        const int e = P[q].b == col ? 0 : 1;
+                        const T un = (e ? v[q][1] : v[q][0]) +
+                                     prolong_cell<D, W, T>(Nc, gc, fld, P[q].i + e, P[q].j, P[q].k);
+                        if (e)
+                            v[q][1] = un;
+                        else
+                            v[q][0] = un;
+                        sm[tl.uoff[l] + col * np + P[q].t] = un;
+                    }
+                }
+                barrier(l);
+                for (int it = 0; it < post; ++it) {
+                    half(l, 1, false);
+                    half(l, 0, false);
+                }
+                store_nat(l, T(0));
+            }
         }
     }
+    __syncthreads();
 }
 
 template <int D, bool W, typename T>
@@ -768,16 +944,19 @@ __global__ void __launch_bounds__(1024) k_mg_tail(const __grid_constant__ TailLe
     {
         T* u0 = sm + tl.uoff[0];
         T* f0 = sm + tl.foff[0];
-        for (int c = tid; c < n0; c += nt) {
-            f0[c] = fg[c];
-            u0[c] = zero_start ? T(0) : ug[c];
-        }
+        for (int c = tid; c < n0; c += nt) f0[c] = fg[c];
+        if (!zero_start)
+            for (int t = tid; t < (n0 >> 1); t += nt) {
+                const TailPair<D> p = tail_pair<D>(tl, 0, t);
+                u0[p.b * (n0 >> 1) + t] = ug[2 * t];
+                u0[(1 - p.b) * (n0 >> 1) + t] = ug[2 * t + 1];
+            }
     }
     __syncthreads();
     tail_solve<D, W, T>(tl, sm, fld, sigma, zero_start, pre, post, sweeps, red);
     {
-        const T* u0 = sm + tl.uoff[0];
-        for (int c = tid; c < n0; c += nt) ug[c] = u0[c];
+        const T* r0 = sm + tl.noff[0];
+        for (int c = tid; c < n0; c += nt) ug[c] = r0[c];
     }
 }
 
@@ -1190,7 +1369,7 @@ __global__ void __launch_bounds__(1024) k_mg_cluster(const __grid_constant__ Clu
 #pragma unroll
             for (int e = 0; e < 2; ++e)
                 cp[e] = coarse_dist ? dplane(l + 1, cl.uoff[l + 1], Kc[e])
-                                    : cluster.map_shared_rank(tailbase + cl.tail.uoff[0], 0) + Kc[e] * (n0c * n1c);
+                                    : cluster.map_shared_rank(tailbase + cl.tail.noff[0], 0) + Kc[e] * (n0c * n1c);
             T acc = T(0);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
@@ -1240,6 +1419,240 @@ __global__ void __launch_bounds__(1024) k_mg_cluster(const __grid_constant__ Clu
         T* dst = ug + (long long)r * n;
         for (int c = tid; c < n; c += nt) dst[c] = u0[c];
     }
+}
+
+// ---- one leg of a 2-D V-cycle level in one launch ---------------------------------
+// A 2-D level fits the L2 many times over and is bound by the launches of its half
+// sweeps.  Here a block holds a tile of the level with a halo and runs a whole leg
+// on it: the down leg every pre-smoothing half sweep, the residual and its
+// restriction, the up leg the prolongation and every post-smoothing half sweep.
+// The valid region shrinks by one cell per half sweep, so the halo is as deep as
+// the leg has of them, and neighbouring tiles form the cells they share twice:
+// the same point operators on the same values, so the result is that of the
+// per-level kernels.  A thread owns one pair of cells (one of each colour) of tile
+// and halo and keeps f and u of it in registers; shared memory holds u, one array
+// per colour.  A leg reads one array of u and writes another (a tile's halo is its
+// neighbour's interior): the down leg writes the level's temporary, the up leg
+// reads that and writes u.  In 3-D the halo of four cells on each side multiplies
+// the work of an 8^3 tile by eight, and the launches win (64^3: 147 us per
+// application of P_S with them, 325 with legs).
+struct LegArgs {
+    Geo gf, gc;
+    int fld0;
+    int t0, t1;   // tile (even)
+    int hn, R1;   // pairs per row, rows of tile and halo
+    int H;        // halo (even)
+    int m0;       // tiles along x
+    FastDiv dh, dc0, dm0;  // hn, t0 / 2, m0
+};
+
+__device__ __forceinline__ int leg_wrap(int x, int n) {
+    if (x < 0) x += n;
+    while (x >= n) x -= n;
+    return x;
+}
+
+template <bool W, typename T>
+struct LegPair {
+    int t, px, ly;      // entry, pair in the row, row
+    int x, y;           // grid cell of the pair's even cell (wrapped on periodic axes)
+    int b;              // colour of the even cell
+    int m[2];           // distance of the two cells from the region's edge
+    unsigned ok[2];
+    int adj[2];
+    bool in, tile;      // a pair of the grid; of the tile itself
+    T f[2], v[2], dinv[2];
+    __device__ __forceinline__ LegPair(const LegArgs& a, int bx, int by, int fld, T sigma, T kh2, T inv) {
+        t = threadIdx.x;
+        ly = fdiv(t, a.dh);
+        px = t - ly * a.hn;
+        const Geo& g = a.gf;
+        const int gx = bx * a.t0 - a.H + 2 * px, gy = by * a.t1 - a.H + ly;
+        in = ly < a.R1;
+        tile = in && 2 * px >= a.H && 2 * px < a.H + a.t0 && ly >= a.H && ly < a.H + a.t1 && gx < g.n0 && gy < g.n1;
+        if (W && (((g.wall & 1) && (gx < 0 || gx >= g.n0)) || ((g.wall & 2) && (gy < 0 || gy >= g.n1)))) in = false;
+        x = leg_wrap(gx, g.n0);
+        y = leg_wrap(gy, g.n1);
+        b = y & 1;
+        const int my = min(ly, a.R1 - 1 - ly);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int lx = 2 * px + e;
+            m[e] = in ? min(my, min(lx, 2 * a.hn - 1 - lx)) : -1;
+            ok[e] = 0x3Fu;
+            adj[e] = 0;
+            dinv[e] = inv;
+            f[e] = v[e] = T(0);
+            if (W && in) {
+                const WInfo wi = wall_info<2>(g, fld, x + e, y, 0);
+                ok[e] = wi.ident ? 0u : wi.ok;
+                adj[e] = wi.ident ? 4 : wi.adj;  // a wall face: u = f, residual f - u
+                if (wi.ident)
+                    dinv[e] = T(1);
+                else if (wi.adj != 0)
+                    dinv[e] = T(1) / (sigma + kh2 * T(4 - wi.adj));
+            }
+        }
+    }
+    // neighbour sum of cell e of the pair: o = the other colour's array
+    __device__ __forceinline__ T nbr(const LegArgs& a, const T* o, bool odd) const {
+        const T own = odd ? v[0] : v[1];
+        if (!W) return own + o[odd ? t + 1 : t - 1] + o[t + a.hn] + o[t - a.hn];
+        const unsigned k = odd ? ok[1] : ok[0];
+        T s = T(0);
+        if (k & 1u) s += odd ? own : o[t - 1];
+        if (k & 2u) s += odd ? o[t + 1] : own;
+        if (k & 4u) s += o[t - a.hn];
+        if (k & 8u) s += o[t + a.hn];
+        return s;
+    }
+    // the half sweep of one colour on the cells at least mg from the region's edge
+    __device__ __forceinline__ void half(const LegArgs& a, T* su, T kh2, int color, int mg, bool zero) {
+        const int np = a.hn * a.R1;
+        const bool odd = b != color;
+        if ((odd ? m[1] : m[0]) >= mg) {
+            const T nb = zero ? T(0) : nbr(a, su + (1 - color) * np, odd);
+            const T un = ((odd ? f[1] : f[0]) + kh2 * nb) * (odd ? dinv[1] : dinv[0]);
+            if (odd)
+                v[1] = un;
+            else
+                v[0] = un;
+            su[color * np + t] = un;
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void put(const LegArgs& a, T* su) const {
+        const int np = a.hn * a.R1;
+        if (!in) return;
+        su[b * np + t] = v[0];
+        su[(1 - b) * np + t] = v[1];
+    }
+};
+
+template <typename T>
+struct LegT2;
+template <>
+struct LegT2<float> {
+    using type = float2;
+};
+template <>
+struct LegT2<double> {
+    using type = double2;
+};
+template <typename T>
+__device__ __forceinline__ void leg_ld(const T* p, T (&v)[2]) {
+    const typename LegT2<T>::type q = *reinterpret_cast<const typename LegT2<T>::type*>(p);
+    v[0] = q.x;
+    v[1] = q.y;
+}
+template <typename T>
+__device__ __forceinline__ void leg_st(T* p, const T (&v)[2]) {
+    typename LegT2<T>::type q;
+    q.x = v[0];
+    q.y = v[1];
+    *reinterpret_cast<typename LegT2<T>::type*>(p) = q;
+}
+
+template <bool W, typename T>
+__global__ void __launch_bounds__(1024) k_leg_down(const __grid_constant__ LegArgs a, const T* __restrict__ uin,
+                                                   const T* __restrict__ f, T* __restrict__ uout, T* __restrict__ fc,
+                                                   T sigma, T kh2, T inv, int pre) {
+    pdl_start();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* su = reinterpret_cast<T*>(smem_raw);  // u per colour, then the residual
+    const int np = a.hn * a.R1;
+    T* R = su + 2 * np;
+    const int by = fdiv(blockIdx.x, a.dm0), bx = (int)blockIdx.x - by * a.m0, cmp = blockIdx.y;
+    const int fld = field_of(a.fld0, cmp);
+    const long long off = (long long)cmp * a.gf.ncell;
+    LegPair<W, T> p(a, bx, by, fld, sigma, kh2, inv);
+    const long long c = off + p.x + (long long)a.gf.n0 * p.y;
+    const bool zero = uin == nullptr;
+    if (p.in) leg_ld(f + c, p.f);
+    if (!zero) {
+        if (p.in) leg_ld(uin + c, p.v);
+        p.put(a, su);
+        __syncthreads();
+    }
+    const int s0 = zero ? 0 : 1;  // a zero start reads no neighbours in its first half sweep
+    for (int it = 0; it < pre; ++it) {
+        p.half(a, su, kh2, 0, 2 * it + s0, zero && it == 0);
+        p.half(a, su, kh2, 1, 2 * it + 1 + s0, false);
+    }
+    if (p.tile) leg_st(uout + c, p.v);
+    // residual of the tile's cells (with walls also one cell around it, for the
+    // full weighting along a normal component's axis)
+    T res[2] = {T(0), T(0)};
+    const int need = a.H - (W ? 1 : 0);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        if (p.m[e] < need) continue;
+        const int col = e ? 1 - p.b : p.b;
+        const T nb = p.nbr(a, su + (1 - col) * np, e == 1);
+        if (W && p.ok[e] == 0u)
+            res[e] = p.f[e] - p.v[e];
+        else
+            res[e] = p.f[e] - (sigma * p.v[e] - kh2 * (nb + T(p.adj[e] - 4) * p.v[e]));
+    }
+    if (p.t < np) {
+        if (W) {
+            R[2 * p.t] = res[0];
+            R[2 * p.t + 1] = res[1];
+        } else {
+            R[p.t] = res[0] + res[1];  // the two children in x of one coarse cell
+        }
+    }
+    __syncthreads();
+    const int c0 = a.t0 >> 1, c1 = a.t1 >> 1;
+    if (p.t >= c0 * c1) return;
+    const int iy = fdiv(p.t, a.dc0), ix = p.t - iy * c0;
+    const int x = bx * a.t0 + 2 * ix, y = by * a.t1 + 2 * iy;  // first child
+    if (x >= a.gf.n0 || y >= a.gf.n1) return;
+    const int r0 = (a.H >> 1) + ix + a.hn * (a.H + 2 * iy);  // its pair
+    T acc = T(0);
+    if (!W) {
+        acc = (R[r0] + R[r0 + a.hn]) * T(0.25);
+    } else {
+        const bool nx = (a.gf.wall & 1) && fld == 0, ny = (a.gf.wall & 2) && fld == 1;
+        if (!(nx && x == 0) && !(ny && y == 0)) {
+            const T* q = R + 2 * r0;
+            for (int i = nx ? -1 : 0; i < 2; ++i)
+                for (int j = ny ? -1 : 0; j < 2; ++j)
+                    acc += (nx && i != 0 ? T(0.25) : T(0.5)) * (ny && j != 0 ? T(0.25) : T(0.5)) * q[i + 2 * a.hn * j];
+        }
+    }
+    fc[(long long)cmp * a.gc.ncell + (x >> 1) + (long long)a.gc.n0 * (y >> 1)] = acc;
+}
+
+template <bool W, typename T>
+__global__ void __launch_bounds__(1024) k_leg_up(const __grid_constant__ LegArgs a, const T* __restrict__ uin,
+                                                 const T* __restrict__ uc, const T* __restrict__ f,
+                                                 T* __restrict__ uout, T sigma, T kh2, T inv, int post) {
+    pdl_start();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* su = reinterpret_cast<T*>(smem_raw);
+    const int by = fdiv(blockIdx.x, a.dm0), bx = (int)blockIdx.x - by * a.m0, cmp = blockIdx.y;
+    const int fld = field_of(a.fld0, cmp);
+    const long long off = (long long)cmp * a.gf.ncell;
+    LegPair<W, T> p(a, bx, by, fld, sigma, kh2, inv);
+    const long long c = off + p.x + (long long)a.gf.n0 * p.y;
+    if (p.in) {
+        leg_ld(f + c, p.f);
+        leg_ld(uin + c, p.v);
+        // the first half sweep overwrites colour 1 without reading it
+        const T d = prolong_cell<2, W, T>(uc + (long long)cmp * a.gc.ncell, a.gc, fld, p.x + p.b, p.y, 0);
+        if (p.b)
+            p.v[1] += d;
+        else
+            p.v[0] += d;
+        p.put(a, su);
+    }
+    __syncthreads();
+    for (int it = 0; it < post; ++it) {
+        p.half(a, su, kh2, 1, 2 * it + 1, false);
+        p.half(a, su, kh2, 0, 2 * it + 2, false);
+    }
+    if (p.tile) leg_st(uout + c, p.v);
 }
 
 // q = -D y - hd ; qr = rhs_scale * q
@@ -1559,29 +1972,6 @@ void mg_prolong_correct(const Geo& gf, const Geo& gc, T* u, const T* uc, int C, 
     IBR_CHECK_LAUNCH();
 }
 
-template <typename T>
-void mg_coarse_solve(const Geo& g, T* u, const T* f, int C, int fld0, double sigma, double kappa, int sweeps,
-                     cudaStream_t s) {
-    T kh2 = (T)(kappa / (g.h * g.h));
-    size_t sm = 2 * (size_t)g.ncell * sizeof(T);
-    int nt = g.ncell >= 1024 ? 1024 : (int)((g.ncell + 31) / 32 * 32);
-    ProfScope ps(KID_COARSE, s, 2.0 * C * g.ncell * sizeof(T));
-    const FastDiv d0 = make_fastdiv(g.n0), d1 = make_fastdiv(g.n1);
-    const T inv = g.d == 3 ? rbgs_inv_diag<3, T>((T)sigma, kh2) : rbgs_inv_diag<2, T>((T)sigma, kh2);
-    if (g.d == 3) {
-        if (g.wall)
-            k_coarse<3, true, T><<<C, nt, sm, s>>>(u, f, g, fld0, (T)sigma, kh2, inv, sweeps, d0, d1);
-        else
-            k_coarse<3, false, T><<<C, nt, sm, s>>>(u, f, g, fld0, (T)sigma, kh2, inv, sweeps, d0, d1);
-    } else {
-        if (g.wall)
-            k_coarse<2, true, T><<<C, nt, sm, s>>>(u, f, g, fld0, (T)sigma, kh2, inv, sweeps, d0, d1);
-        else
-            k_coarse<2, false, T><<<C, nt, sm, s>>>(u, f, g, fld0, (T)sigma, kh2, inv, sweeps, d0, d1);
-    }
-    IBR_CHECK_LAUNCH();
-}
-
 // the tail kernels' shared-memory limit, raised once per device (function
 // attributes belong to the device that is current when they are set)
 template <typename T>
@@ -1600,7 +1990,7 @@ void mg_set_attributes() {
 template <typename T>
 static size_t tail_smem(const Geo* lev, int l0, int L) {
     size_t n = 0;
-    for (int l = l0; l < L; ++l) n += 2 * (size_t)lev[l].ncell;
+    for (int l = l0; l < L; ++l) n += 3 * (size_t)lev[l].ncell;
     return n * sizeof(T);
 }
 
@@ -1625,6 +2015,8 @@ TailLevels make_tail(const Geo* lev, int lt, int L, double sigma, double kappa) 
         tl.uoff[q] = off;
         off += (int)lev[lt + q].ncell;
         tl.foff[q] = off;
+        off += (int)lev[lt + q].ncell;
+        tl.noff[q] = off;
         off += (int)lev[lt + q].ncell;
         tl.dh[q] = make_fastdiv(lev[lt + q].n0 / 2);
         tl.d0[q] = make_fastdiv(lev[lt + q].n0);
@@ -1787,10 +2179,75 @@ void rb_launch_half(const Geo& g, int C, T* us, const T* fs, T kh2, T inv, int c
     IBR_CHECK_LAUNCH();
 }
 
+// halo of the down leg (with walls the restriction needs the residual one cell
+// further out) and of the up leg; even, so that pairs stay pairs
+inline int leg_halo_down(const Geo& g, bool zero, int pre) {
+    return (2 * pre + (zero ? 0 : 1) + (g.wall ? 1 : 0) + 1) & ~1;
+}
+inline int leg_halo_up(int post) { return 2 * post; }
+
+// 16 x 16 tiles: enough blocks and a short critical path on small levels, 2.3 times
+// the tile's own cells with the halo of a 2-sweep leg (32 x 32 tiles form 1.6 times
+// and measured within 2 % of them, 512^2 included)
+constexpr int LEG_TILE = 16;
+inline LegArgs leg_args(const Geo& gf, const Geo& gc, int fld0, int H) {
+    LegArgs a;
+    a.gf = gf;
+    a.gc = gc;
+    a.fld0 = fld0;
+    a.H = H;
+    a.t0 = std::min(LEG_TILE, gf.n0);
+    a.t1 = std::min(LEG_TILE, gf.n1);
+    a.hn = a.t0 / 2 + H;
+    a.R1 = a.t1 + 2 * H;
+    a.m0 = (gf.n0 + a.t0 - 1) / a.t0;
+    a.dh = make_fastdiv(a.hn);
+    a.dc0 = make_fastdiv(a.t0 / 2);
+    a.dm0 = make_fastdiv(a.m0);
+    return a;
+}
+inline dim3 leg_grid(const LegArgs& a, int C) {
+    return dim3((unsigned)(a.m0 * ((a.gf.n1 + a.t1 - 1) / a.t1)), (unsigned)C);
+}
+inline int leg_block(const LegArgs& a) { return (a.hn * a.R1 + 31) / 32 * 32; }
+
+// whether a level runs its legs in one launch each
+inline bool leg_ok(const Geo& g, int pre, int post) {
+    return mg_leg_level(g) && pre >= 1 && post >= 1 && pre <= 3 && post <= 3 && g.n0 >= 8 && g.n1 >= 8;
+}
+template <typename T>
+bool leg_aligned(const T* a, const T* b, const T* c) {
+    return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c) % (2 * sizeof(T))) == 0;
+}
+
+template <typename T>
+void leg_down(const Geo& gf, const Geo& gc, const T* uin, const T* f, T* uout, T* fc, int C, int fld0, double sigma,
+              double kappa, int pre, cudaStream_t s) {
+    const LegArgs a = leg_args(gf, gc, fld0, leg_halo_down(gf, uin == nullptr, pre));
+    const T kh2 = (T)(kappa / (gf.h * gf.h)), sg = (T)sigma, inv = rbgs_inv_diag<2, T>(sg, kh2);
+    ProfScope ps(KID_RBGS, s, (2.25 + (uin ? 1.0 : 0.0)) * C * gf.ncell * sizeof(T));
+    const size_t sm = (size_t)(gf.wall ? 4 : 3) * a.hn * a.R1 * sizeof(T);
+    launch_k(gf.wall ? k_leg_down<true, T> : k_leg_down<false, T>, leg_grid(a, C), dim3(leg_block(a)), sm, s, a, uin, f,
+             uout, fc, sg, kh2, inv, pre);
+    IBR_CHECK_LAUNCH();
+}
+
+template <typename T>
+void leg_up(const Geo& gf, const Geo& gc, const T* uin, const T* uc, const T* f, T* uout, int C, int fld0, double sigma,
+            double kappa, int post, cudaStream_t s) {
+    const LegArgs a = leg_args(gf, gc, fld0, leg_halo_up(post));
+    const T kh2 = (T)(kappa / (gf.h * gf.h)), sg = (T)sigma, inv = rbgs_inv_diag<2, T>(sg, kh2);
+    ProfScope ps(KID_RBGS, s, 3.25 * C * gf.ncell * sizeof(T));
+    const size_t sm = (size_t)2 * a.hn * a.R1 * sizeof(T);
+    launch_k(gf.wall ? k_leg_up<true, T> : k_leg_up<false, T>, leg_grid(a, C), dim3(leg_block(a)), sm, s, a, uin, uc, f,
+             uout, sg, kh2, inv, post);
+    IBR_CHECK_LAUNCH();
+}
+
 template <typename T>
 void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, int C, int fld0, double sigma,
                double kappa, bool zero_start, int pre, int post, int coarse_sweeps, cudaStream_t s, T* rb_u,
-               T* rb_f, T* rb_u1, T* rb_f1) {
+               T* rb_f, T* rb_u1, T* rb_f1, T* const* Wt) {
     auto Fl = [&](int l) -> const T* { return l == 0 ? F0 : Fw[l]; };
     // periodic 3-D: the finest level and the next in red-black split layout
     // (conversions folded into the first and last half sweeps of each)
@@ -1800,15 +2257,34 @@ void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, in
     for (int l = 0; l < 2; ++l)
         split_l[l] = L > l + 1 && (long long)C * lev[l].ncell < (1LL << 31) &&
                      rb_split_ok<T>(lev[l], Fl(l), U[l], rbu[l], rbf[l], l > 0 || zero_start, pre, post);
-    auto split = [&](int l) { return l < 2 && split_l[l]; };
+    // a level runs as two legs where it is small enough for launch latency to
+    // bound it (a level in split layout never is, unless legs take it)
+    auto legs = [&](int l) {
+        return Wt && Wt[l] && l + 1 < L && leg_ok(lev[l], pre, post) && leg_aligned<T>(Fl(l), U[l], Wt[l]);
+    };
+    auto split = [&](int l) { return l < 2 && split_l[l] && !legs(l); };
     // periodic 3-D: the coarse levels on one thread-block cluster per field
     ClusterLevels cl;
     int top = 0;
     const int want = cluster_choice(lev, L, C, sizeof(T));
     const bool use_cluster =
         want != -2 && cluster_plan<T>(lev, L, sigma, kappa, want, top, cl) && cluster_ok<T>();
-    const int lt = use_cluster ? top : tail_start<T>(lev, L);
+    int lt = use_cluster ? top : tail_start<T>(lev, L);
+    // The tail runs on one SM per field.  Where its larger levels can run on many
+    // and that is faster, they do: FP64 sweeps, at two operations per clock and SM,
+    // from 32^2 and 8^3 up (FP64 P_S on 64^2 76 us, 135 with that level in the
+    // tail; on 64^3 387, 421), and FP32 with walls, whose boundary rules cost
+    // registers, from 32^2 up (64^2 61 us, 70); FP32 on periodic grids keeps them.
+    const long long most = sizeof(T) == 8 ? (lev[0].d == 2 ? 1024 : 512)
+                                          : (lev[0].d == 2 && lev[0].wall ? 1024 : MG_TAIL_MAX_CELLS);
+    if (!use_cluster)
+        while (lt + 1 < L && lev[lt].ncell > most && (lev[0].d == 3 || legs(lt))) ++lt;
     for (int l = 0; l < lt; ++l) {
+        if (legs(l)) {
+            leg_down<T>(lev[l], lev[l + 1], l > 0 || zero_start ? (const T*)nullptr : (const T*)U[l], Fl(l), Wt[l],
+                        Fw[l + 1], C, fld0, sigma, kappa, pre, s);
+            continue;
+        }
         if (split(l)) {
             const Geo& g = lev[l];
             T* ru = rbu[l];
@@ -1873,7 +2349,8 @@ void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, in
         TailLevels tl = make_tail<T>(lev, lt, L, sigma, kappa);
         size_t sm = tail_smem<T>(lev, lt, L);
         long long n0 = lev[lt].ncell;
-        int nt = n0 >= 2048 ? 1024 : (int)(((n0 + 1) / 2 + 31) / 32 * 32);
+        // one thread per pair of cells, at most TAIL_NP pairs each
+        int nt = n0 >= 2048 ? 1024 : (int)((n0 / 2 + 31) / 32 * 32);
         if (nt < 32) nt = 32;
         ProfScope ps(KID_COARSE, s, 2.0 * C * n0 * sizeof(T));
         mg_set_attributes<T>();
@@ -1895,6 +2372,11 @@ void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, in
         IBR_CHECK_LAUNCH();
     }
     for (int l = lt - 1; l >= 0; --l) {
+        if (legs(l)) {
+            leg_up<T>(lev[l], lev[l + 1], (const T*)Wt[l], (const T*)U[l + 1], Fl(l), U[l], C, fld0, sigma, kappa, post,
+                      s);
+            continue;
+        }
         if (split(l)) {
             const Geo& g = lev[l];
             T* ru = rbu[l];
@@ -2067,12 +2549,11 @@ void wall_lift(const Geo& g, int a, int side, const double* data, double* b, dou
     template void mg_residual_restrict<T>(const Geo&, const Geo&, const T*, const T*, T*, int, int, double, \
                                           double, cudaStream_t);                                          \
     template void mg_prolong_correct<T>(const Geo&, const Geo&, T*, const T*, int, int, cudaStream_t);    \
-    template void mg_coarse_solve<T>(const Geo&, T*, const T*, int, int, double, double, int, cudaStream_t); \
     template void mg_set_attributes<T>();                                                                   \
     template void mg_tune_smoother<T>(const Geo&, int, cudaStream_t);                                       \
     template void mg_tune_cluster<T>(const Geo*, int, T* const*, T* const*, int, int, cudaStream_t);          \
     template void mg_vcycle<T>(const Geo*, int, T* const*, T* const*, const T*, int, int, double, double, bool, \
-                               int, int, int, cudaStream_t, T*, T*, T*, T*);                                \
+                               int, int, int, cudaStream_t, T*, T*, T*, T*, T* const*);                                \
     template void ps_divergence<T>(const Geo&, const T*, const T*, T*, double, T*, cudaStream_t);         \
     template void ps_finish<T>(const Geo&, const T*, const T*, const T*, T*, double, double, cudaStream_t);
 IBR_INST(double)
