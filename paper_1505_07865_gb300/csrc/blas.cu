@@ -962,118 +962,238 @@ __global__ void k_df_scale(long long n, const double* __restrict__ inv_norm, con
     }
 }
 
-// ---- modified Gram-Schmidt over the FP64 basis: one pass per basis vector ---
-// Step i of MGS subtracts the projection on V_i from w and, in the same pass
-// over the entries, forms the dot of the updated w with V_{i+1} (or, after
-// the last vector, |w|^2): two FP64 FMAs per entry.  The pass for V_0 only
-// forms V_0 . w, the last pass scales w into V_K.  A pass leaves one partial
-// sum per block; the next pass reduces them itself, in every block and in a
-// fixed order (bitwise the same value everywhere, no separate reduction
-// kernel), and block 0 records the coefficient.
-constexpr int MG_BLOCKS = 5 * 152;  // five resident blocks of 256 threads per SM (<= 48 registers)
+// ---- modified Gram-Schmidt over the FP64 basis, MGS_B vectors per pass ------------
+// A pass subtracts from w the projections on one block of basis vectors and, in
+// the same sweep over the entries, forms the dots of the updated w with the next
+// block (after the last one, |w|^2).  Within a block the sequential
+// coefficients follow from the dots by the block's Gram matrix, whose strictly
+// lower part L holds the (rounding-size) dots of its vectors with each other:
+//   h_q = V_q . (w - sum_{r<q} h_r V_r) = a_q - sum_{r<q} L_qr h_r,
+// modified Gram-Schmidt with its products regrouped (the inverse compact WY form:
+// Swirydowicz, Langou, Ananthan, Yang, Thomas, "Low synchronization Gram-Schmidt
+// and generalized minimal residual algorithms", 2021).  L is formed where a vector
+// is made: the last pass, which has the block in registers, also forms its dots
+// with the remainder.  Two FP64 FMAs per entry and vector, as with one vector per
+// pass, but w moves once per block: 18 bytes per entry and vector instead of 32.
+// The FP64 pipe bounds it (89 % busy; 128^3: 28.5 us per vector, 48 with one vector
+// per pass, whose loads and sums did not overlap; whole solves at 128^3 61.3 ->
+// 52.9 ms, 192^3 299 -> 254 ms, and 512^2 53.0 -> 41.8 ms against CGS2).  A pass leaves one partial sum
+// per block of threads and dot; the next pass sums them itself, in every block and
+// in a fixed order (bitwise the same value everywhere), and block 0 records the
+// coefficients.
+constexpr int MGS_B = 8;
+constexpr int MGS_BLOCKS = 2 * 152;  // two resident blocks of 256 threads per SM (<= 128 registers)
 
-// the sum of the previous pass' partials (fixed order), broadcast to the block
-__device__ __forceinline__ double mgs_prev(const double* __restrict__ pin, int nblk, double* sh) {
-    double x = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) x += pin[b];
-    double v[1] = {x};
-    block_sum<1>(v, sh);
-    return sh[0];
+// out[q] = sum of v[q] over the block (the block is synchronised after it).
+// Summed through shared memory: with shuffles alone every value would take five
+// FP64 additions of every warp.
+template <int NQ>
+__device__ __forceinline__ void mgs_block_sums(const double (&v)[NQ], double* buf, double* out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) buf[q * RED_THREADS + threadIdx.x] = v[q];
+    __syncthreads();
+    for (int q = wid; q < NQ; q += RED_THREADS / 32) {
+        double x = 0.0;
+#pragma unroll
+        for (int u = 0; u < RED_THREADS / 32; ++u) x += buf[q * RED_THREADS + u * 32 + lane];
+        x = warp_sum(x);
+        if (lane == 0) out[q] = x;
+    }
+    __syncthreads();
 }
 
-// mode 0: pout = V_0 . w.  mode 1: h = sum(pin), hcol[i] = h (block 0),
-// w -= h V_i, pout = V_{i+1} . w (i + 1 < K) or w . w (i + 1 == K).
-// n2: entry pairs (n even, a zero pad entry), V_i: rows of ld doubles.
-__global__ void __launch_bounds__(RED_THREADS, 5) k_mgs_step(long long n2, const double* __restrict__ Vi,
-                                                          const double* __restrict__ Vn, double* __restrict__ w,
-                                                          const double* __restrict__ pin, double* __restrict__ pout,
-                                                          double* __restrict__ hcol, int mode) {
-    pdl_start();
-    __shared__ double sh[1];
-    double h = 0.0;
-    if (mode == 1) {
-        h = mgs_prev(pin, gridDim.x, sh);
-        if (blockIdx.x == 0 && threadIdx.x == 0) *hcol = h;
+// the sums of a pass' partials pin[q * nblk + blk], q < nq, into out (synchronised)
+__device__ __forceinline__ void mgs_collect(const double* __restrict__ pin, int nblk, int nq, double* out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int q = wid; q < nq; q += RED_THREADS / 32) {
+        double x = 0.0;
+        for (int b = lane; b < nblk; b += 32) x += pin[q * nblk + b];
+        x = warp_sum(x);
+        if (lane == 0) out[q] = x;
     }
-    const double2* v2 = reinterpret_cast<const double2*>(Vi);
-    const double2* n2p = reinterpret_cast<const double2*>(Vn);  // NULL: the norm of w
-    double2* w2 = reinterpret_cast<double2*>(w);
-    // two pairs per trip (p and p + stride): their loads are issued together
-    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    for (; p + stride < n2; p += 2 * stride) {
-        const long long q = p + stride;
-        double2 x = w2[p], y = w2[q];
-        if (mode == 1) {
-            const double2 v = __ldcs(v2 + p), vq = __ldcs(v2 + q);  // last use of V_i in this step
-            x.x = fma(-h, v.x, x.x);
-            x.y = fma(-h, v.y, x.y);
-            y.x = fma(-h, vq.x, y.x);
-            y.y = fma(-h, vq.y, y.y);
-            w2[p] = x;
-            w2[q] = y;
-        }
-        const double2 u = mode == 0 ? __ldg(v2 + p) : (n2p ? __ldg(n2p + p) : x);
-        const double2 uq = mode == 0 ? __ldg(v2 + q) : (n2p ? __ldg(n2p + q) : y);
-        a0 = fma(u.x, x.x, a0);
-        a1 = fma(u.y, x.y, a1);
-        b0 = fma(uq.x, y.x, b0);
-        b1 = fma(uq.y, y.y, b1);
-    }
-    if (p < n2) {
-        double2 x = w2[p];
-        if (mode == 1) {
-            const double2 v = __ldcs(v2 + p);
-            x.x = fma(-h, v.x, x.x);
-            x.y = fma(-h, v.y, x.y);
-            w2[p] = x;
-        }
-        const double2 u = mode == 0 ? __ldg(v2 + p) : (n2p ? __ldg(n2p + p) : x);
-        a0 = fma(u.x, x.x, a0);
-        a1 = fma(u.y, x.y, a1);
-    }
-    double v[1] = {(a0 + a1) + (b0 + b1)};
-    block_sum<1>(v, sh);
-    if (threadIdx.x == 0) pout[blockIdx.x] = sh[0];
+    __syncthreads();
 }
 
-// nu^2 = sum(pin) = |w|^2; st[2] = nu^2, st[3] = 1 / nu (block 0);
-// V_K = w / nu, out32 (first n32 entries, float) its FP32 copy
-__global__ void __launch_bounds__(RED_THREADS, 5) k_mgs_norm(long long n2, const double* __restrict__ w,
-                                                          const double* __restrict__ pin, double* __restrict__ st,
-                                                          double* __restrict__ vout, float* __restrict__ out32,
-                                                          long long n32) {
+// w -= the projections on the NS vectors at Vs (their dots with w in pin; L: rows
+// of MGS_B of the block's Gram matrix; coefficients to hcol), then the dots with the
+// ND vectors at Vd into pout.  ND == 0: the last pass, which forms the dots with
+// the NS vectors themselves (unless their block is full: the new vector then
+// begins the next) and, as number NS, |w|^2.  n2: entry pairs, ld2: their stride
+// between vectors.  The counts are template parameters: FMAs switched off by a
+// predicate take the FP64 pipe as long as the others.
+template <int NS, int ND>
+__global__ void __launch_bounds__(RED_THREADS, 2)
+    k_mgs_block(long long n2, long long ld2, const double2* __restrict__ Vs, const double2* __restrict__ Vd,
+                double2* __restrict__ w, const double* __restrict__ L, const double* __restrict__ pin,
+                double* __restrict__ pout, double* __restrict__ hcol) {
     pdl_start();
-    __shared__ double sh[1];
-    __shared__ double inv_s;
-    const double nu2 = mgs_prev(pin, gridDim.x, sh);
-    if (threadIdx.x == 0) {
-        const double nu = sqrt(fmax(nu2, 0.0));
-        inv_s = nu > 0.0 ? 1.0 / nu : 0.0;
-        if (blockIdx.x == 0) {
-            st[0] = nu2;
-            st[1] = 0.0;
-            st[2] = fmax(nu2, 0.0);
-            st[3] = inv_s;
+    constexpr bool LAST = ND == 0, GRAM = LAST && NS < MGS_B;
+    constexpr int NQ = LAST ? NS + 1 : ND;
+    __shared__ double buf[NQ * RED_THREADS];
+    __shared__ double sums[MGS_B + 1];
+    double h[NS > 0 ? NS : 1];
+    if constexpr (NS > 0) {
+        mgs_collect(pin, gridDim.x, NS, sums);
+        if (threadIdx.x < 32) {
+            const int q = threadIdx.x;
+            double x = q < NS ? sums[q] : 0.0;
+            for (int r = 0; r + 1 < NS; ++r) {
+                const double hr = __shfl_sync(0xffffffffu, x, r);
+                if (q > r && q < NS) x = fma(-L[q * MGS_B + r], hr, x);
+            }
+            if (q < NS) {
+                sums[q] = x;
+                if (blockIdx.x == 0) hcol[q] = x;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NS; ++q) h[q] = sums[q];
+    }
+    double acc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n2; p += (long long)gridDim.x * blockDim.x) {
+        double2 x = w[p];
+        double2 v[NS > 0 ? NS : 1], d[ND > 0 ? ND : 1];
+#pragma unroll
+        for (int q = 0; q < NS; ++q) v[q] = __ldcs(Vs + q * ld2 + p);
+#pragma unroll
+        for (int q = 0; q < ND; ++q) d[q] = __ldg(Vd + q * ld2 + p);
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            x.x = fma(-h[q], v[q].x, x.x);
+            x.y = fma(-h[q], v[q].y, x.y);
+        }
+        if (NS > 0) w[p] = x;
+#pragma unroll
+        for (int q = 0; q < ND; ++q) acc[q] = fma(d[q].y, x.y, fma(d[q].x, x.x, acc[q]));
+        if constexpr (GRAM) {
+#pragma unroll
+            for (int q = 0; q < NS; ++q) acc[q] = fma(v[q].y, x.y, fma(v[q].x, x.x, acc[q]));
+        }
+        if constexpr (LAST) acc[NS] = fma(x.y, x.y, fma(x.x, x.x, acc[NS]));
+    }
+    mgs_block_sums<NQ>(acc, buf, sums);
+    if (threadIdx.x < NQ) pout[threadIdx.x * gridDim.x + blockIdx.x] = sums[threadIdx.x];
+}
+
+using MgsPass = void (*)(long long, long long, const double2*, const double2*, double2*, const double*, const double*,
+                         double*, double*);
+// the pass that subtracts ns vectors (0 or MGS_B, or any number in the last pass, nd == 0)
+inline MgsPass mgs_pass(int ns, int nd) {
+    static const MgsPass dots[2][MGS_B] = {
+        {k_mgs_block<0, 1>, k_mgs_block<0, 2>, k_mgs_block<0, 3>, k_mgs_block<0, 4>, k_mgs_block<0, 5>, k_mgs_block<0, 6>,
+         k_mgs_block<0, 7>, k_mgs_block<0, 8>},
+        {k_mgs_block<8, 1>, k_mgs_block<8, 2>, k_mgs_block<8, 3>, k_mgs_block<8, 4>, k_mgs_block<8, 5>, k_mgs_block<8, 6>,
+         k_mgs_block<8, 7>, k_mgs_block<8, 8>}};
+    static const MgsPass last[MGS_B] = {k_mgs_block<1, 0>, k_mgs_block<2, 0>, k_mgs_block<3, 0>, k_mgs_block<4, 0>,
+                                        k_mgs_block<5, 0>, k_mgs_block<6, 0>, k_mgs_block<7, 0>, k_mgs_block<8, 0>};
+    return nd == 0 ? last[ns - 1] : dots[ns ? 1 : 0][nd - 1];
+}
+
+// Column j of the Hessenberg matrix from the coefficients h[0..j] and nr = |w_perp|,
+// the Givens rotations applied, the new one formed, res_out = |g[j + 1]| (one
+// block; the rotations run on one thread, on copies in shared memory, since their
+// operands would otherwise come one memory latency after the other)
+__device__ void givens_column(double* H, int ldh, const double* h, double nr, int j, double* cs, double* sn, double* gv,
+                              double* res_out, double* sm) {
+    double *c = sm, *s = sm + 128, *col = sm + 256;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+        col[i] = h[i];
+        if (i < j) {
+            c[i] = cs[i];
+            s[i] = sn[i];
         }
     }
     __syncthreads();
-    const double inv = inv_s;
+    if (threadIdx.x == 0) {
+        double a = col[0];
+        for (int i = 0; i < j; ++i) {
+            const double b = col[i + 1];
+            col[i] = c[i] * a + s[i] * b;
+            a = -s[i] * a + c[i] * b;
+        }
+        const double r = hypot(a, nr);
+        const double cj = r > 0.0 ? a / r : 1.0, sj = r > 0.0 ? nr / r : 0.0;
+        col[j] = r;
+        cs[j] = cj;
+        sn[j] = sj;
+        const double gj = gv[j];
+        gv[j] = cj * gj;
+        gv[j + 1] = -sj * gj;
+        *res_out = fabs(sj * gj);
+    }
+    __syncthreads();
+    double* out = H + (long long)j * ldh;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) out[i] = col[i];
+    if (threadIdx.x == 0) out[j + 1] = 0.0;
+}
+
+// nu^2 = |w|^2 = sum number ng of pin; st[2] = nu^2, st[3] = 1 / nu; V_k = w / nu, out32
+// (first n32 entries, float) its FP32 copy; its Gram row grow[q] = sum q / nu
+// (q < ng); block 0 also finishes the Hessenberg column (givens_column, j = k - 1)
+__global__ void __launch_bounds__(RED_THREADS) k_mgs_norm(long long n2, const double* __restrict__ w,
+                                                          const double* __restrict__ pin, int nblk, int ns, int ng,
+                                                          double* __restrict__ st, double* __restrict__ vout,
+                                                          float* __restrict__ out32, long long n32,
+                                                          double* __restrict__ grow, double* __restrict__ H, int ldh,
+                                                          const double* __restrict__ h, int j, double* cs, double* sn,
+                                                          double* gv, double* res_out) {
+    pdl_start();
+    __shared__ double sums[MGS_B + 1];
+    __shared__ double piece[2];
+    __shared__ double sm[3 * 128];
+    mgs_collect(pin + ns * nblk, nblk, 1, sums + ns);
+    if (threadIdx.x == 0) {
+        const double nu = sqrt(fmax(sums[ns], 0.0));
+        piece[0] = nu;
+        piece[1] = nu > 0.0 ? 1.0 / nu : 0.0;
+    }
+    __syncthreads();
+    const double nu = piece[0], inv = piece[1];
     const double2* w2 = reinterpret_cast<const double2*>(w);
     double2* v2 = reinterpret_cast<double2*>(vout);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n2;
-         p += (long long)gridDim.x * blockDim.x) {
-        const double2 x = w2[p];
-        const double2 y = make_double2(x.x * inv, x.y * inv);
-        v2[p] = y;
+    // four entries per trip: one 16-byte store of the FP32 copy
+    const long long stride = (long long)gridDim.x * blockDim.x, nq = n2 / 2;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nq; t += stride) {
+        const double2 a = w2[2 * t], b = w2[2 * t + 1];
+        const double2 x = make_double2(a.x * inv, a.y * inv), y = make_double2(b.x * inv, b.y * inv);
+        v2[2 * t] = x;
+        v2[2 * t + 1] = y;
         if (out32) {
-            const long long i = 2 * p;
-            if (i + 1 < n32)
-                *reinterpret_cast<float2*>(out32 + i) = make_float2((float)y.x, (float)y.y);
-            else if (i < n32)
-                out32[i] = (float)y.x;
+            const long long i = 4 * t;
+            if (i + 4 <= n32) {
+                *reinterpret_cast<float4*>(out32 + i) = make_float4((float)x.x, (float)x.y, (float)y.x, (float)y.y);
+            } else {
+                const double e[4] = {x.x, x.y, y.x, y.y};
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (i + q < n32) out32[i + q] = (float)e[q];
+            }
         }
+    }
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0 && (n2 & 1)) {
+            const double2 a = w2[n2 - 1];
+            const double2 x = make_double2(a.x * inv, a.y * inv);
+            v2[n2 - 1] = x;
+            const long long i = 2 * (n2 - 1);
+            if (out32 && i < n32) out32[i] = (float)x.x;
+            if (out32 && i + 1 < n32) out32[i + 1] = (float)x.y;
+        }
+        if (ng > 0) {
+            mgs_collect(pin, nblk, ng, sums);
+            if (threadIdx.x < ng) grow[threadIdx.x] = sums[threadIdx.x] * inv;
+        }
+        if (threadIdx.x == 0) {
+            st[0] = sums[ns];
+            st[1] = 0.0;
+            st[2] = fmax(sums[ns], 0.0);
+            st[3] = inv;
+        }
+        givens_column(H, ldh, h, nu, j, cs, sn, gv, res_out, sm);
     }
 }
 
@@ -1475,32 +1595,39 @@ void scale_df(long long n, long long n_real, const double* inv_norm, const doubl
 }
 
 void mgs_orthonormalize(long long n, const double* V, long long ld, int k, double* w, double* vout, float* out32,
-                        long long n32, double* partial, double* h, double* st, cudaStream_t s) {
-    if ((n & 1) || (ld & 1) || k < 1)
-        throw Error{IBR_EINVAL, "modified Gram-Schmidt: even length and leading dimension, k >= 1 required"};
-    if ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(vout)) & 15)
-        throw Error{IBR_EINVAL, "modified Gram-Schmidt: V, w and vout must be 16-byte aligned"};
-    const long long n2 = n / 2;
+                        long long n32, double* partial, double* gram, double* h, double* st, double* H, int ldh,
+                        double* cs, double* sn, double* gv, double* res_out, cudaStream_t s) {
+    if ((n & 1) || (ld & 1) || k < 1 || k > 127)
+        throw Error{IBR_EINVAL, "modified Gram-Schmidt: even length and leading dimension, 1 <= k <= 127 required"};
+    if ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(vout) |
+         reinterpret_cast<uintptr_t>(out32)) & 15)
+        throw Error{IBR_EINVAL, "modified Gram-Schmidt: V, w, vout and out32 must be 16-byte aligned"};
+    const long long n2 = n / 2, ld2 = ld / 2;
+    // at least four pairs per thread, so that a block's sums do not outweigh its sweep
+    const int grid = (int)std::max<long long>(1, std::min<long long>(MGS_BLOCKS, n2 / (4 * RED_THREADS)));
     double* pa = partial;
-    double* pb = partial + MG_BLOCKS;
-    {
-        ProfScope ps(KID_MDOT, s, 2.0 * n * 8.0);
-        launch_k(k_mgs_step, dim3(MG_BLOCKS), dim3(RED_THREADS), 0, s, n2, V, (const double*)nullptr, w,
-                 (const double*)nullptr, pa, (double*)nullptr, 0);
-        IBR_CHECK_LAUNCH();
-    }
-    for (int i = 0; i < k; ++i) {
-        // V_i, V_{i+1} (or the norm) and w read, w written
-        ProfScope ps(KID_UPD_MDOT, s, (i + 1 < k ? 4.0 : 3.0) * n * 8.0, 4.0 * n);
-        const double* Vn = i + 1 < k ? V + (long long)(i + 1) * ld : nullptr;
-        launch_k(k_mgs_step, dim3(MG_BLOCKS), dim3(RED_THREADS), 0, s, n2, V + (long long)i * ld, Vn, w,
-                 (const double*)pa, pb, h + i, 1);
+    double* pb = partial + (MGS_B + 1) * MGS_BLOCKS;
+    const double2* V2 = reinterpret_cast<const double2*>(V);
+    double2* w2 = reinterpret_cast<double2*>(w);
+    const int nb = (k + MGS_B - 1) / MGS_B;
+    for (int p = 0; p <= nb; ++p) {
+        // pass p: subtract block p - 1, dots with block p (p == nb: the norm)
+        const int i0 = (p - 1) * MGS_B, ns = p > 0 ? std::min(MGS_B, k - i0) : 0;
+        const int nd = p < nb ? std::min(MGS_B, k - p * MGS_B) : 0;
+        ProfScope ps(p ? KID_UPD_MDOT : KID_MDOT, s, (ns + nd + (p ? 2.0 : 1.0)) * n * 8.0,
+                     2.0 * n * (ns + (p < nb ? nd : 1 + (ns < MGS_B ? ns : 0))));
+        launch_k(mgs_pass(ns, nd), dim3(grid), dim3(RED_THREADS), 0, s, n2, ld2, V2 + (p > 0 ? i0 : 0) * ld2,
+                 V2 + (long long)p * MGS_B * (p < nb ? ld2 : 0), w2, (const double*)(gram + (p > 0 ? i0 : 0) * MGS_B),
+                 (const double*)pa, pb, h + (p > 0 ? i0 : 0));
         IBR_CHECK_LAUNCH();
         std::swap(pa, pb);
     }
+    const int ns = k - (nb - 1) * MGS_B;
     ProfScope ps(KID_UPD_NORM, s, 2.0 * n * 8.0 + (out32 ? 4.0 * n32 : 0.0));
-    launch_k(k_mgs_norm, dim3(MG_BLOCKS), dim3(RED_THREADS), 0, s, n2, (const double*)w, (const double*)pa, st, vout,
-             out32, n32);
+    const int gridn = (int)std::max<long long>(1, std::min<long long>(4 * 152, n2 / (2 * RED_THREADS)));
+    launch_k(k_mgs_norm, dim3(gridn), dim3(RED_THREADS), 0, s, n2, (const double*)w, (const double*)pa, grid, ns,
+             k % MGS_B ? ns : 0, st, vout, out32, n32, gram + (long long)k * MGS_B, H, ldh, (const double*)h, k - 1, cs,
+             sn, gv, res_out);
     IBR_CHECK_LAUNCH();
 }
 

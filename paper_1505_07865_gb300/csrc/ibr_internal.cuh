@@ -402,12 +402,17 @@ struct __align__(8) dflt {
 // Modified Gram-Schmidt of w against the FP64 basis V_0..V_{k-1} (rows of
 // ld doubles) and V_k = the normalised remainder into vout, with an FP32 copy
 // of its first n32 entries (out32, may be NULL): h[0..k) the coefficients,
-// st[2] = |w_perp|^2, st[3] its inverse square root, st[1] = 0.  k + 2
-// launches, two FP64 FMAs per entry and basis vector; w is overwritten.  n and
-// ld even (entries past the system length are a zero pad of w and of every
-// basis vector), V, w, vout 16-byte aligned; partial holds 2 * 760 doubles.
+// st[2] = |w_perp|^2, st[3] its inverse square root, st[1] = 0; column k - 1 of
+// H with its Givens rotation as arnoldi_column does it.  Eight vectors per pass
+// and two FP64 FMAs per entry and vector; w is overwritten.  n and ld even
+// (entries past the system length are a zero pad of w and of every basis vector),
+// V, w, vout, out32 16-byte aligned, 1 <= k <= 127; partial holds 2 * 9 * 304
+// doubles, gram 8 (k + 1): the dots of the basis vectors of one block of eight,
+// kept from step to step of a cycle.
+constexpr int MGS_GRAM = 8;
 void mgs_orthonormalize(long long n, const double* V, long long ld, int k, double* w, double* vout, float* out32,
-                        long long n32, double* partial, double* h, double* st, cudaStream_t s);
+                        long long n32, double* partial, double* gram, double* h, double* st, double* H, int ldh,
+                        double* cs, double* sn, double* gv, double* res_out, cudaStream_t s);
 // cgs_orthonormalize of the outer FGMRES basis, pipelined on bulk copies: V
 // is FP64 or (df) double-float, 8 bytes per entry either way; w is FP64 on
 // entry (double-float: converted in place, w's contents are consumed); the

@@ -209,7 +209,7 @@ struct ibr_grid {
     double* xc = nullptr;  // the iterate at the start of a cycle that goes on after its first residual
     double *H = nullptr, *cs = nullptr, *sn = nullptr, *gv = nullptr, *yv = nullptr;
     double *h1 = nullptr, *h2 = nullptr, *sc = nullptr, *partial = nullptr, *shift = nullptr, *means = nullptr;
-    double *hk2 = nullptr, *st = nullptr;
+    double *hk2 = nullptr, *st = nullptr, *gram = nullptr;
     int* wait_err = nullptr;    // set by a pipelined Gram-Schmidt pass whose wait timed out
     double* host_sc = nullptr;  // pinned
     double* FT = nullptr;
@@ -594,7 +594,7 @@ void free_markers(ibr_grid* G) {
 
 void free_outer(ibr_grid* G) {
     double** ps[] = {&G->V, &G->Z, &G->b, &G->x, &G->w, &G->H, &G->cs, &G->sn, &G->gv, &G->yv,
-                     &G->h1, &G->h2, &G->sc, &G->partial, &G->shift, &G->means, &G->hk2, &G->st, &G->vk64, &G->xc};
+                     &G->h1, &G->h2, &G->sc, &G->partial, &G->shift, &G->means, &G->hk2, &G->st, &G->vk64, &G->xc, &G->gram};
     for (double** p : ps) dfree(*p);
     dfree(G->wait_err);
     G->m_alloc = 0;
@@ -1155,10 +1155,11 @@ void ensure_outer(ibr_grid* G, int m) {
     G->h2 = dalloc<double>(m + 1);
     G->hk2 = dalloc<double>(m + 2);
     G->st = dalloc<double>(4);
+    G->gram = dalloc<double>((size_t)MGS_GRAM * (m + 2));
     G->sc = dalloc<double>(8);
     G->wait_err = dalloc<int>(1);
     IBR_CUDA_TRY(cudaMemsetAsync(G->wait_err, 0, sizeof(int), G->stream));
-    G->partial = dalloc<double>((size_t)RED_BLOCKS * std::max(m + 1, 4));
+    G->partial = dalloc<double>((size_t)RED_BLOCKS * std::max(m + 1, 10));
     G->shift = dalloc<double>(4);
     G->means = dalloc<double>(4);
     G->len_alloc = len;
@@ -1223,27 +1224,23 @@ void project_solution(ibr_grid* G, double* x) {
 }
 
 // The outer Arnoldi orthogonalisation, over the FP64 basis in both
-// precisions.  Systems of at least ARN_MGS_MIN_LEN entries: modified
-// Gram-Schmidt (two FP64 FMAs per entry and basis vector; on this part the
-// FP64 pipe, not HBM, bounds these passes, and MGS halves their work).
-// Smaller systems: classical Gram-Schmidt with reorthogonalisation (CGS2, four
-// FMAs) pipelined on bulk copies, three launches per step instead of MGS's
-// k + 2 (there the passes are short and launch latency decides).
-// IBR_ARNOLDI in the environment forces one: "mgs", "cgs2", or "df" (CGS2 over
-// a double-float basis: pairs of floats, a 48-bit significand, arithmetic on
-// the FP32 pipe; for comparison).
+// precisions: modified Gram-Schmidt, eight vectors per pass (blas.cu).  On this
+// part the FP64 pipe bounds it, with two FMAs per entry and basis vector;
+// classical Gram-Schmidt with reorthogonalisation (CGS2) needs four, and its eight
+// launches per step are no gain on small systems either, where the blocked form has
+// k / 8 + 2 (solves at 64^3 34.1 -> 27.1 ms, 256^2 13.7 -> 12.6, 64^2 6.0 -> 5.6).
+// IBR_ARNOLDI in the environment forces one: "mgs", "cgs2" (pipelined on bulk
+// copies), or "df" (CGS2 over a double-float basis: pairs of floats, a 48-bit
+// significand, arithmetic on the FP32 pipe; for comparison).
 enum { ARN_MGS = 0, ARN_CGS2 = 1, ARN_DF = 2 };
-constexpr long long ARN_MGS_MIN_LEN = 2000000;
-int arnoldi_kind(long long len) {
-    static const int forced = [] {
+int arnoldi_kind() {
+    static const int kind = [] {
         const char* e = std::getenv("IBR_ARNOLDI");
-        if (e && std::string(e) == "mgs") return (int)ARN_MGS;
         if (e && std::string(e) == "cgs2") return (int)ARN_CGS2;
         if (e && std::string(e) == "df") return (int)ARN_DF;
-        return -1;
+        return (int)ARN_MGS;
     }();
-    if (forced >= 0) return forced;
-    return len >= ARN_MGS_MIN_LEN ? (int)ARN_MGS : (int)ARN_CGS2;
+    return kind;
 }
 
 // warm: start from the x already in G->x (time stepping), else from x = 0
@@ -1313,7 +1310,7 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
         // its fluid part is written by the same pass
         float* rs32 = G->precision == IBR_MIXED ? G->pc32->rs : nullptr;
         const long long lp = G->len_pad();
-        const int arn = arnoldi_kind(len);
+        const int arn = arnoldi_kind();
         const bool df = arn == ARN_DF;
         // double-float basis: the preconditioner reads the fluid part from
         // rs32 (mixed) or vk64 (FP64), the constraint part from vk64
@@ -1337,14 +1334,14 @@ int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm
             // the FP64 basis: the preconditioner reads V_{j+1} itself (and, mixed,
             // the FP32 copy of its fluid part in rs32)
             if (arn == ARN_MGS) {
-                mgs_orthonormalize(lp, G->V, lp, j + 1, G->w, Vj + lp, rs32, G->nS, G->partial, G->h1, G->st, s);
+                mgs_orthonormalize(lp, G->V, lp, j + 1, G->w, Vj + lp, rs32, G->nS, G->partial, G->gram, G->h1, G->st,
+                                   G->H, m + 1, G->cs, G->sn, G->gv, G->sc + 3, s);
             } else {
                 cgs_orthonormalize_pipe(df, lp, len, G->V, lp, j + 1, G->w, Vj + lp, rs32, G->nS,
                                         df ? G->vk64 : nullptr, from64, G->partial, G->h1, G->h2, G->hk2, G->st,
                                         G->wait_err, s);
+                arnoldi_column(G->H, m + 1, G->h1, G->h2, G->st + 2, j, G->cs, G->sn, G->gv, G->sc + 3, G->sc + 4, s);
             }
-            arnoldi_column(G->H, m + 1, G->h1, arn == ARN_MGS ? nullptr : G->h2, G->st + 2, j, G->cs, G->sn, G->gv,
-                           G->sc + 3, G->sc + 4, s);
             info.iters++;
             double est = read_scalar(G, G->sc + 3);
             info.rel_res_est = est / bnorm;
@@ -1540,7 +1537,7 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
     double t = 0.0;
     // outer FGMRES
     t += pg(8.0 * (m + 1) * lp) + pg(8.0 * m * len) + 4 * pg(8.0 * len) + pg(8.0 * lp);
-    t += 8.0 * ((m + 1) * (m + 1) + 8 * (m + 2)) + pg(8.0 * RED_BLOCKS * std::max(m + 1, 4));
+    t += 8.0 * ((m + 1) * (m + 1) + 8 * (m + 2)) + pg(8.0 * RED_BLOCKS * std::max(m + 1, 10));
     // preconditioner: coarse multigrid levels (d stacked fields, u and f)
     Geo c = g;
     while (Multigrid<float>::can_coarsen(c)) {
