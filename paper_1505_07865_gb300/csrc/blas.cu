@@ -1132,7 +1132,7 @@ __device__ void givens_column(double* H, int ldh, const double* h, double nr, in
 }
 
 // nu^2 = |w|^2 = sum number ng of pin; st[2] = nu^2, st[3] = 1 / nu; V_k = w / nu, out32
-// (first n32 entries, float) its FP32 copy; its Gram row grow[q] = sum q / nu
+// (first n32 entries, float) its FP32 copy, out64 its entries from64 .. n64 - 1; its Gram row grow[q] = sum q / nu
 // (q < ng); block 0 also finishes the Hessenberg column (givens_column, j = k - 1)
 __global__ void __launch_bounds__(RED_THREADS) k_mgs_norm(long long n2, const double* __restrict__ w,
                                                           const double* __restrict__ pin, int nblk, int ns, int ng,
@@ -1140,7 +1140,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_norm(long long n2, const do
                                                           float* __restrict__ out32, long long n32,
                                                           double* __restrict__ grow, double* __restrict__ H, int ldh,
                                                           const double* __restrict__ h, int j, double* cs, double* sn,
-                                                          double* gv, double* res_out) {
+                                                          double* gv, double* res_out, double* __restrict__ out64,
+                                                          long long from64, long long n64) {
     pdl_start();
     __shared__ double sums[MGS_B + 1];
     __shared__ double piece[2];
@@ -1174,6 +1175,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_norm(long long n2, const do
             }
         }
     }
+    if (out64 && blockIdx.x == gridDim.x - 1)
+        for (long long i = from64 + threadIdx.x; i < n64; i += blockDim.x) out64[i - from64] = w[i] * inv;
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0 && (n2 & 1)) {
             const double2 a = w2[n2 - 1];
@@ -1445,6 +1448,100 @@ __global__ void k_subtract_means_v(long long m, T* __restrict__ x, const double*
     }
 }
 
+// ---- the vector passes of the inner solve (up to INNER_MAX directions) --------
+template <int K, typename T>
+__global__ void __launch_bounds__(256) k_inner_direction(long long n, T* __restrict__ w, const T* __restrict__ r,
+                                                         const T* __restrict__ V, long long ld,
+                                                         const double* __restrict__ y, int vec) {
+    pdl_start();
+    T c[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) c[i] = (T)pdl_ld(y + i);
+    const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (vec) {
+        for (long long q = t0; q < n / 4; q += stride) {
+            Q4<T> a = reinterpret_cast<const Q4<T>*>(w)[q];
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const Q4<T> v = reinterpret_cast<const Q4<T>*>(i == 0 ? r : V + (i - 1) * ld)[q];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) a.v[e] -= c[i] * v.v[e];
+            }
+            reinterpret_cast<Q4<T>*>(w)[q] = a;
+        }
+    } else {
+        for (long long q = t0; q < n; q += stride) {
+            T a = w[q];
+#pragma unroll
+            for (int i = 0; i < K; ++i) a -= c[i] * (i == 0 ? r : V + (i - 1) * ld)[q];
+            w[q] = a;
+        }
+    }
+}
+
+// blockIdx.y: block of m entries; the last of a block's thread blocks sums its mean
+template <int K, typename T>
+__global__ void __launch_bounds__(256) k_inner_combine(long long m, const T* __restrict__ Z, long long ld,
+                                                       const double* __restrict__ y, T* __restrict__ x, int d,
+                                                       double* __restrict__ means, double* __restrict__ partial,
+                                                       unsigned* __restrict__ ticket, int vec) {
+    pdl_start();
+    T c[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) c[i] = (T)pdl_ld(y + i);
+    const int cmp = blockIdx.y;
+    Z += (long long)cmp * m;
+    x += (long long)cmp * m;
+    const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    T s0 = T(0), e0 = T(0), s1 = T(0), e1 = T(0);
+    const bool sum = means != nullptr && cmp < d;
+    if (vec) {
+        for (long long q = t0; q < m / 4; q += stride) {
+            Q4<T> a;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a.v[e] = T(0);
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const Q4<T> v = reinterpret_cast<const Q4<T>*>(Z + i * ld)[q];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) a.v[e] += c[i] * v.v[e];
+            }
+            reinterpret_cast<Q4<T>*>(x)[q] = a;
+            if (sum) {
+                add_keep(a.v[0], s0, e0);
+                add_keep(a.v[1], s1, e1);
+                add_keep(a.v[2], s0, e0);
+                add_keep(a.v[3], s1, e1);
+            }
+        }
+    } else {
+        for (long long q = t0; q < m; q += stride) {
+            T a = T(0);
+#pragma unroll
+            for (int i = 0; i < K; ++i) a += c[i] * Z[i * ld + q];
+            x[q] = a;
+            if (sum) add_keep(a, s0, e0);
+        }
+    }
+    if (!sum) return;
+    __shared__ double o[1];
+    __shared__ bool last;
+    double v[1] = {((double)s0 + (double)s1) + ((double)e0 + (double)e1)};
+    block_sum<1>(v, o);
+    if (threadIdx.x == 0) {
+        partial[cmp * gridDim.x + blockIdx.x] = o[0];
+        __threadfence();
+        last = atomicInc(ticket + cmp, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    double t = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) t += __ldcg(partial + cmp * gridDim.x + b);
+    t = warp_sum(t);
+    if (threadIdx.x == 0) means[cmp] = t / (double)m;
+}
+
 inline bool vec16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 template <typename T>
 inline bool vec16_basis(const T* V, long long ld) { return vec16(V) && (ld * (long long)sizeof(T)) % 16 == 0; }
@@ -1596,7 +1693,8 @@ void scale_df(long long n, long long n_real, const double* inv_norm, const doubl
 
 void mgs_orthonormalize(long long n, const double* V, long long ld, int k, double* w, double* vout, float* out32,
                         long long n32, double* partial, double* gram, double* h, double* st, double* H, int ldh,
-                        double* cs, double* sn, double* gv, double* res_out, cudaStream_t s) {
+                        double* cs, double* sn, double* gv, double* res_out, double* out64, long long from64,
+                        long long n64, cudaStream_t s) {
     if ((n & 1) || (ld & 1) || k < 1 || k > 127)
         throw Error{IBR_EINVAL, "modified Gram-Schmidt: even length and leading dimension, 1 <= k <= 127 required"};
     if ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(vout) |
@@ -1627,7 +1725,7 @@ void mgs_orthonormalize(long long n, const double* V, long long ld, int k, doubl
     const int gridn = (int)std::max<long long>(1, std::min<long long>(4 * 152, n2 / (2 * RED_THREADS)));
     launch_k(k_mgs_norm, dim3(gridn), dim3(RED_THREADS), 0, s, n2, (const double*)w, (const double*)pa, grid, ns,
              k % MGS_B ? ns : 0, st, vout, out32, n32, gram + (long long)k * MGS_B, H, ldh, (const double*)h, k - 1, cs,
-             sn, gv, res_out);
+             sn, gv, res_out, out64, from64, n64);
     IBR_CHECK_LAUNCH();
 }
 
@@ -1723,6 +1821,32 @@ void combine(long long n, const Tz* Z, long long ld, int k, const double* y, T* 
     IBR_CHECK_LAUNCH();
 }
 template <typename T>
+void inner_direction(long long n, T* w, const T* r, const T* V, long long ld, int k, const double* y, cudaStream_t s) {
+    ProfScope ps(KID_UPD_NORM, s, (k + 2.0) * n * sizeof(T));
+    const int vec = n % 4 == 0 && vec16(r) && vec16(w) && vec16_basis(V, ld) ? 1 : 0;
+    const dim3 grid((unsigned)std::min<long long>(8 * 152, n / (vec ? 1024 : 256) + 1));
+    auto go = [&](auto* kern) { launch_k(kern, grid, dim3(256), 0, s, n, w, r, V, ld, y, vec); };
+    if (k == 1) go(k_inner_direction<1, T>);
+    else if (k == 2) go(k_inner_direction<2, T>);
+    else if (k == 3) go(k_inner_direction<3, T>);
+    else throw Error{IBR_EINVAL, "inner_direction: 1 to 3 vectors"};
+    IBR_CHECK_LAUNCH();
+}
+template <typename T>
+void inner_combine(long long m, int nc, const T* Z, long long ld, int k, const double* y, T* x, int d, double* means,
+                   double* partial, unsigned* ticket, cudaStream_t s) {
+    ProfScope ps(KID_COMBINE, s, (k + 1.0) * m * nc * sizeof(T));
+    const int vec = m % 4 == 0 && vec16(x) && vec16_basis(Z, ld) ? 1 : 0;
+    const dim3 grid((unsigned)std::min<long long>(152, m / (vec ? 1024 : 256) + 1), (unsigned)nc);
+    auto go = [&](auto* kern) { launch_k(kern, grid, dim3(256), 0, s, m, Z, ld, y, x, d, means, partial, ticket, vec); };
+    if (k == 1) go(k_inner_combine<1, T>);
+    else if (k == 2) go(k_inner_combine<2, T>);
+    else if (k == 3) go(k_inner_combine<3, T>);
+    else if (k == 4) go(k_inner_combine<4, T>);
+    else throw Error{IBR_EINVAL, "inner_combine: 1 to 4 directions"};
+    IBR_CHECK_LAUNCH();
+}
+template <typename T>
 void block_means(long long m, int C, const T* x, double* partial, double* out, cudaStream_t s) {
     ProfScope ps(KID_BLOCK_MEANS, s, (double)m * C * sizeof(T));
     if (m % 4 == 0 && vec16(x))
@@ -1782,6 +1906,9 @@ void hess_solve(const double* H, int ldh, const double* gv, int k, double* y, cu
     template void update_norm2<T>(long long, const T*, long long, int, const double*, T*, double*, double*,     \
                                   cudaStream_t);                                                                \
     template void norm2<T>(long long, const T*, double*, double*, cudaStream_t);                                \
+    template void inner_direction<T>(long long, T*, const T*, const T*, long long, int, const double*, cudaStream_t); \
+    template void inner_combine<T>(long long, int, const T*, long long, int, const double*, T*, int, double*, double*, \
+                                   unsigned*, cudaStream_t);                                                    \
     template void block_means<T>(long long, int, const T*, double*, double*, cudaStream_t);                     \
     template void block_means_acc<T>(long long, int, const T*, double*, double*, cudaStream_t);                 \
     template void subtract_means<T>(long long, int, T*, const double*, cudaStream_t);

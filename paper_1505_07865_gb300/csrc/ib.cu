@@ -268,44 +268,100 @@ __global__ void k_spread_gather(long long F, const long long* __restrict__ face,
     y[face[f]] += scale * s;
 }
 
-// one warp per marker; lanes stride the KW^D support of each component
+// one warp per marker and component; lanes stride the KW^D support
+template <int D, int KW, typename T>
+__device__ __forceinline__ T interp_warp(const Geo& g, int ia, const int* __restrict__ idx, const T* __restrict__ w,
+                                         const T* __restrict__ v) {
+    constexpr int S = D == 3 ? KW * KW * KW : KW * KW;
+    const int lane = threadIdx.x & 31, a = ia % D;
+    const T* va = v + a * g.ncell;
+    const int* id = idx + (long long)ia * D * KW;
+    const T* wt = w + (long long)ia * D * KW;
+    T acc = T(0);
+#pragma unroll
+    for (int c0 = 0; c0 < S; c0 += 32) {
+        const int c = c0 + lane;
+        if (c < S) {
+            const int m0 = c % KW, m1 = (c / KW) % KW, m2 = c / (KW * KW);
+            int cell = id[m0] + g.n0 * id[KW + m1];
+            T t = wt[m0] * wt[KW + m1];
+            if (D == 3) {
+                cell += g.n0 * g.n1 * id[2 * KW + m2];
+                t *= wt[2 * KW + m2];
+            }
+            acc += t * va[cell];
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+
 template <int D, int KW, typename T, typename Tadd>
 __global__ void k_interp(Geo g, int N, const int* __restrict__ idx, const T* __restrict__ w, const T* __restrict__ v,
                          T* __restrict__ out, T sign, const Tadd* __restrict__ add, T add_scale,
                          const double* __restrict__ mean) {
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (warp >= N) return;
-    const int S = D == 3 ? KW * KW * KW : KW * KW;
-    const int ns[3] = {g.n0, g.n1, g.n2};
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        const T* va = v + a * g.ncell;
-        long long ia = (long long)warp * D + a;
-        T acc = T(0);
-        for (int c = lane; c < S; c += 32) {
-            long long cell = 0, stride = 1;
-            T wt = T(1);
-            int cc = c;
-#pragma unroll
-            for (int b = 0; b < D; ++b) {
-                const int m = cc % KW;
-                cc /= KW;
-                long long t = ia * D + b;
-                int j = idx[t * KW + m];
-                cell += j * stride;
-                stride *= ns[b];
-                wt *= w[t * KW + m];
-            }
-            acc += wt * va[cell];
-        }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) {
-            // the weights of a window sum to one: J (v - m) = J v - m
-            T r = sign * (mean ? acc - (T)mean[a] : acc);
-            if (add) r += add_scale * (T)add[ia];
-            out[ia] = r;
-        }
+    const int ia = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (ia >= N * D) return;
+    const T acc = interp_warp<D, KW, T>(g, ia, idx, w, v);
+    if ((threadIdx.x & 31) == 0) {
+        // the weights of a window sum to one: J (v - m) = J v - m
+        T r = sign * (mean ? acc - (T)mean[ia % D] : acc);
+        if (add) r += add_scale * (T)add[ia];
+        out[ia] = r;
+    }
+}
+
+// blocks [0, nsb): spreading, the others interpolation (they share no data)
+template <int D, int KW>
+__global__ void __launch_bounds__(128) k_spread_interp(Geo g, int N, int nsb, long long F,
+                                                       const long long* __restrict__ face, const int* __restrict__ off,
+                                                       const int* __restrict__ ent_m, const double* __restrict__ ew,
+                                                       const double* __restrict__ lam, double* __restrict__ y,
+                                                       double scale, const int* __restrict__ idx,
+                                                       const double* __restrict__ w, const double* __restrict__ v,
+                                                       double* __restrict__ out, double sign,
+                                                       const double* __restrict__ mean) {
+    pdl_start();
+    if ((int)blockIdx.x < nsb) {
+        const long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+        if (f >= F) return;
+        double s = 0.0;
+        const int e1 = off[f + 1];
+        for (int e = off[f]; e < e1; ++e) s += ew[e] * lam[ent_m[e]];
+        y[face[f]] += scale * s;
+        return;
+    }
+    const int ia = (((int)blockIdx.x - nsb) * (int)blockDim.x + (int)threadIdx.x) >> 5;
+    if (ia >= N * D) return;
+    const double acc = interp_warp<D, KW, double>(g, ia, idx, w, v);
+    if ((threadIdx.x & 31) == 0) out[ia] = sign * (mean ? acc - mean[ia % D] : acc);
+}
+
+// block c < d: component c of lam converted and summed; block d: U
+template <typename T>
+__global__ void __launch_bounds__(1024) k_lam_out(int d, int N, const T* __restrict__ lam, double* __restrict__ z, int nU,
+                                                  const double* __restrict__ U, double scale,
+                                                  double* __restrict__ shift) {
+    __shared__ double sm[32];
+    const int c = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (c == d) {
+        for (int i = threadIdx.x; i < nU; i += blockDim.x) z[(long long)N * d + i] = U[i];
+        return;
+    }
+    double s = 0.0;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        const double x = (double)lam[(long long)i * d + c];
+        z[(long long)i * d + c] = x;
+        s += x;
+    }
+    if (!shift) return;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sm[wid] = s;
+    __syncthreads();
+    if (wid == 0) {
+        s = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) shift[c] = scale * s;
     }
 }
 
@@ -479,7 +535,7 @@ void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign,
             double add_scale, const double* mean) {
     const T* w = sizeof(T) == 8 ? reinterpret_cast<const T*>(md.w64) : reinterpret_cast<const T*>(md.w32);
     int threads = 128;
-    int blocks = grid_1d((long long)md.N * 32, threads);
+    int blocks = grid_1d((long long)md.N * g.d * 32, threads);
     const int kw = g.kw;
     ProfScope ps(KID_INTERP, s,
                  (double)md.N * g.d * ((g.d == 3 ? kw * kw * kw : kw * kw) * sizeof(T) + g.d * kw * sizeof(T) + sizeof(T)));
@@ -500,6 +556,30 @@ void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign,
     }
     IBR_CHECK_LAUNCH();
 }
+
+void spread_interp(const Geo& g, const MarkerData& md, const double* lam, double* y, double scale, const double* v,
+                   double* out, double sign, const double* mean, cudaStream_t s) {
+    const int kw = g.kw, nsb = md.F > 0 ? grid_1d(md.F, 128) : 0;
+    const int nib = grid_1d((long long)md.N * g.d * 32, 128);
+    ProfScope ps(KID_SPREAD, s, (double)md.F * 28.0 + (double)md.E * 20.0 +
+                                    (double)md.N * g.d * 8.0 * ((g.d == 3 ? kw * kw * kw : kw * kw) + g.d * kw + 1));
+    auto* k = g.d == 3 ? (kw == 6 ? k_spread_interp<3, 6> : k_spread_interp<3, 4>)
+                       : (kw == 6 ? k_spread_interp<2, 6> : k_spread_interp<2, 4>);
+    launch_k(k, dim3((unsigned)(nsb + nib)), dim3(128), 0, s, g, md.N, nsb, md.F, (const long long*)md.face,
+             (const int*)md.off, (const int*)md.ent_m, (const double*)md.ent_w64, lam, y, scale, (const int*)md.idx,
+             (const double*)md.w64, v, out, sign, mean);
+    IBR_CHECK_LAUNCH();
+}
+
+template <typename T>
+void lam_out(int d, int N, const T* lam, double* z, int nU, const double* U, double scale, double* shift, cudaStream_t s) {
+    ProfScope ps(KID_LAMSUM, s, (double)N * d * (8 + sizeof(T)));
+    const int nt = N >= 1024 ? 1024 : (N + 31) / 32 * 32;
+    k_lam_out<T><<<d + (nU > 0 ? 1 : 0), nt, 0, s>>>(d, N, lam, z, nU, U, scale, shift);
+    IBR_CHECK_LAUNCH();
+}
+template void lam_out<double>(int, int, const double*, double*, int, const double*, double, double*, cudaStream_t);
+template void lam_out<float>(int, int, const float*, double*, int, const double*, double, double*, cudaStream_t);
 
 template <typename T>
 void lam_sum(int d, int N, const T* lam, double scale, double* shift, cudaStream_t s) {

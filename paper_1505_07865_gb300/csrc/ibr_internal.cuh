@@ -101,6 +101,10 @@ __device__ __forceinline__ void pdl_start() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 bool pdl_enabled();
+// A value that the predecessor wrote, read at the very start of a kernel: through a
+// const __restrict__ pointer such a load may be scheduled ahead of the wait in
+// pdl_start when no branch lies between them; a volatile one is not.
+__device__ __forceinline__ double pdl_ld(const double* p) { return *reinterpret_cast<const volatile double*>(p); }
 
 // Bulk asynchronous copies into shared memory with completion counted on an
 // mbarrier (the producer / consumer pipelines of the tensor-core products and
@@ -248,6 +252,22 @@ inline int grid_1d(long long work, int block) {
 template <typename T>
 void stokes_apply(const Geo& g, const T* x, T* y, double sigma, double eta, const double* shift_dev,
                   cudaStream_t s);
+// the same on a periodic grid from x in FP32 or FP64, FP64 arithmetic and result; z
+// (may be NULL): x in FP64
+template <typename Ti>
+void stokes_apply_from(const Geo& g, const Ti* x, double* y, double* z, double sigma, double eta, const double* shift_dev,
+                       cudaStream_t s);
+// Step nw < INNER_MAX of an inner GMRES solve with the orthogonal, not normalised
+// basis V_0 = r, V_1 .. V_nw (at Vv, stride ld): w = L z with sigma, eta as above and its
+// Hessenberg column (hs, nv: state of the solve).  y: the coefficients of the basis
+// vectors in w (for the next direction) or, fin, of the directions z in the
+// solution (w is then not written).  partial: INNER_BLOCKS * (INNER_MAX + 2)
+// doubles; ticket: zero.
+constexpr int INNER_MAX = 4;
+constexpr int INNER_BLOCKS = 8 * 152;
+template <typename T>
+void stokes_dots(const Geo& g, const T* z, T* w, const T* r, const T* Vv, long long ld, int nw, bool fin, double sigma,
+                 double eta, double* partial, unsigned* ticket, double* hs, double* nv, double* y, cudaStream_t s);
 // The multigrid pieces act on C stacked fields with field codes fld0,
 // fld0 + 1, ... (fld0 == FLD_P: one pressure field), which fix the boundary
 // rule of each field on wall axes.
@@ -364,6 +384,15 @@ void norm2(long long n, const T* w, double* partial, double* out, cudaStream_t s
 template <typename T, typename Tz>
 void combine(long long n, const Tz* Z, long long ld, int k, const double* y, T* x, bool accumulate,
              cudaStream_t s);
+// w -= y_0 r + sum_{0 < i < k} y_i V_i, the V_i at V (stride ld); 1 <= k < INNER_MAX, y on the device
+template <typename T>
+void inner_direction(long long n, T* w, const T* r, const T* V, long long ld, int k, const double* y, cudaStream_t s);
+// x = sum_{i < k} y_i Z_i over nc blocks of m entries; means (device, d doubles, or
+// NULL): the means of the first d blocks with their rounding errors kept, as
+// block_means_acc forms them.  partial: 152 * d doubles; ticket: zero
+template <typename T>
+void inner_combine(long long m, int nc, const T* Z, long long ld, int k, const double* y, T* x, int d, double* means,
+                   double* partial, unsigned* ticket, cudaStream_t s);
 // means of C consecutive blocks of length m (partial sums, double), then
 // x_c -= mean_c for the blocks selected by mask
 template <typename T>
@@ -401,8 +430,9 @@ struct __align__(8) dflt {
 };
 // Modified Gram-Schmidt of w against the FP64 basis V_0..V_{k-1} (rows of
 // ld doubles) and V_k = the normalised remainder into vout, with an FP32 copy
-// of its first n32 entries (out32, may be NULL): h[0..k) the coefficients,
-// st[2] = |w_perp|^2, st[3] its inverse square root, st[1] = 0; column k - 1 of
+// of its first n32 entries (out32, may be NULL) and an FP64 one of the entries
+// from64 .. n64 - 1 (out64): h[0..k) the coefficients, st[2] = |w_perp|^2, st[3] its
+// inverse square root, st[1] = 0; column k - 1 of
 // H with its Givens rotation as arnoldi_column does it.  Eight vectors per pass
 // and two FP64 FMAs per entry and vector; w is overwritten.  n and ld even
 // (entries past the system length are a zero pad of w and of every basis vector),
@@ -412,7 +442,8 @@ struct __align__(8) dflt {
 constexpr int MGS_GRAM = 8;
 void mgs_orthonormalize(long long n, const double* V, long long ld, int k, double* w, double* vout, float* out32,
                         long long n32, double* partial, double* gram, double* h, double* st, double* H, int ldh,
-                        double* cs, double* sn, double* gv, double* res_out, cudaStream_t s);
+                        double* cs, double* sn, double* gv, double* res_out, double* out64, long long from64,
+                        long long n64, cudaStream_t s);
 // cgs_orthonormalize of the outer FGMRES basis, pipelined on bulk copies: V
 // is FP64 or (df) double-float, 8 bytes per entry either way; w is FP64 on
 // entry (double-float: converted in place, w's contents are consumed); the
@@ -475,6 +506,14 @@ void spread_gather(const MarkerData& md, const T* lam, T* y, double scale, cudaS
 template <typename T, typename Tadd>
 void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign, const Tadd* add,
             cudaStream_t s, double add_scale, const double* mean = nullptr);
+// The marker part of a product with the system matrix in one launch: y (fluid
+// rows) += scale S lam, out = sign J (v - mean) as spread_gather and interp do them
+void spread_interp(const Geo& g, const MarkerData& md, const double* lam, double* y, double scale, const double* v,
+                   double* out, double sign, const double* mean, cudaStream_t s);
+// lam's N*d entries in FP64 to z, U's nU entries (may be 0) after them, and shift as lam_sum
+// forms it (NULL: not needed); one launch
+template <typename T>
+void lam_out(int d, int N, const T* lam, double* z, int nU, const double* U, double scale, double* shift, cudaStream_t s);
 // shift[a] = scale * sum_i lam[i*d+a]  (double, a < d)
 template <typename T>
 void lam_sum(int d, int N, const T* lam, double scale, double* shift, cudaStream_t s);

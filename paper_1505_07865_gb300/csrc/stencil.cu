@@ -220,73 +220,272 @@ __device__ __forceinline__ long long fx_int(double v, int emax) {
     const long long sg = (long long)((int)hi >> 31);
     return ((long long)(m >> sh) ^ sg) - sg;
 }
-// c 2^(emax - 1081): what one unit of fx_int(., emax) is worth, times c; ok: it is a normal number
-__device__ __forceinline__ double fx_scale(double c, int emax, bool& ok) {
+// The same for FP32 values (the preconditioner's result): 24-bit significands leave
+// 35 bits below, so values within 2^35 of the largest lose nothing.
+__device__ __forceinline__ int fx_exp(float v) { return (__float_as_int(v) >> 23) & 0xff; }
+__device__ __forceinline__ long long fx_int(float v, int emax) {
+    const unsigned b = __float_as_uint(v);
+    const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << 35;
+    const int sh = min(emax - (int)((b >> 23) & 0xff), 63);
+    const long long sg = (long long)((int)b >> 31);
+    return ((long long)(m >> sh) ^ sg) - sg;
+}
+// c times what one unit of fx_int(., emax) is worth; ok: it is a normal number and the
+// sum's values are far enough from the ends of their type's range
+__device__ __forceinline__ double fx_times(double c, int q, bool& ok) {
     const int hi = __double2hiint(c);
-    const int e = ((hi >> 20) & 0x7ff) + emax - 1081;
-    ok = emax >= 128 && emax < 0x7ff && e >= 1 && e < 0x7ff;
+    const int e = ((hi >> 20) & 0x7ff) + q;
+    ok = ok && e >= 1 && e < 0x7ff;
     return __hiloint2double((hi & 0x800fffff) | (e << 20), __double2loint(c));
 }
+template <typename Ti>
+__device__ __forceinline__ double fx_scale(double c, int emax, bool& ok) {
+    if constexpr (sizeof(Ti) == 8) {
+        ok = emax >= 128 && emax < 0x7ff;
+        return fx_times(c, emax - 1081, ok);
+    } else {
+        ok = emax >= 64 && emax < 0xff;
+        return fx_times(c, emax - 185, ok);
+    }
+}
+// the exact FP64 value (an FP32 one through its bits: the conversion instruction
+// runs at the FP64 rate)
+__device__ __forceinline__ double fx_val(double v) { return v; }
+__device__ __forceinline__ double fx_val(float v) {
+    const unsigned b = __float_as_uint(v);
+    const unsigned e = (b >> 23) & 0xff;
+    if (e == 0 || e == 0xff) return (b << 1) ? (double)v : __hiloint2double((int)(b & 0x80000000u), 0);
+    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b >> 3) & 0xfffffu)), (int)(b << 29));
+}
 
-template <int D>
-__global__ void __launch_bounds__(256) k_stokes_fx(const double* __restrict__ x, double* __restrict__ y, Geo g,
-                                                   double sigma, double kh2, double ih,
-                                                   const double* __restrict__ shift) {
-    pdl_start();
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
-    if (i >= g.n0 || j >= g.n1) return;
-    const Nbr n = neighbours<D>(g, i, j, k);
-    const double* p = x + D * g.ncell + n.c;
-    const double pc = *p;
+// rows of cell n: val[a] = sigma v^a - kh2 Lap v^a + (p_c - p_{c-e_a}) ih, val[D] = -div
+template <int D, typename Ti>
+__device__ __forceinline__ void fx_rows(const Ti* __restrict__ x, const Geo& g, const Nbr& n, double sigma, double kh2,
+                                        double ih, double (&val)[D + 1], Ti (&own)[D + 1]) {
+    const Ti* p = x + D * g.ncell + n.c;
+    const Ti pc = *p;
+    const double pd = fx_val(pc);
     const int off[6] = {n.xp, n.xm, n.yp, n.ym, n.zp, n.zm};
-    double uc[D], up[D];  // u_a at the cell's low and high face of axis a
+    Ti up[D];  // u_a at the cell's high face of axis a
     int ed = 0;
+    bool ok;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const double* u = x + a * g.ncell + n.c;
-        double v[2 * D];
-        uc[a] = *u;
-        int em = fx_exp(uc[a]);
+        const Ti* u = x + a * g.ncell + n.c;
+        Ti v[2 * D];
+        const Ti uc = *u;
+        int em = fx_exp(uc);
 #pragma unroll
         for (int q = 0; q < 2 * D; ++q) {
             v[q] = u[off[q]];
             em = max(em, fx_exp(v[q]));
         }
+        own[a] = uc;
         up[a] = v[2 * a];
-        ed = max(ed, max(fx_exp(uc[a]), fx_exp(up[a])));
-        bool ok;
-        const double c = fx_scale(-kh2, em, ok);
-        double val;
+        ed = max(ed, max(fx_exp(uc), fx_exp(up[a])));
+        const double c = fx_scale<Ti>(-kh2, em, ok);
+        double r;
         if (ok) {
-            long long s = -(2 * D) * fx_int(uc[a], em);
+            long long s = -(2 * D) * fx_int(uc, em);
 #pragma unroll
             for (int q = 0; q < 2 * D; ++q) s += fx_int(v[q], em);
-            val = __ll2double_rn(s) * c;
+            r = __ll2double_rn(s) * c;
         } else {
-            double s = v[0] + v[1] + v[2] + v[3];
-            if (D == 3) s += v[2 * D - 2] + v[2 * D - 1];
-            val = -kh2 * (s - 2.0 * D * uc[a]);
+            double s = (double)v[0] + (double)v[1] + (double)v[2] + (double)v[3];
+            if (D == 3) s += (double)v[2 * D - 2] + (double)v[2 * D - 1];
+            r = -kh2 * (s - 2.0 * D * (double)uc);
         }
-        if (sigma != 0.0) val = fma(sigma, uc[a], val);
-        val = fma(pc - p[off[2 * a + 1]], ih, val);
-        if (shift) val += shift[a];
-        y[a * g.ncell + n.c] = val;
+        if (sigma != 0.0) r = fma(sigma, fx_val(uc), r);
+        val[a] = fma(pd - fx_val(p[off[2 * a + 1]]), ih, r);
     }
-    bool ok;
-    const double c = fx_scale(-ih, ed, ok);
-    double val;
+    own[D] = pc;
+    const double c = fx_scale<Ti>(-ih, ed, ok);
     if (ok) {
         long long s = 0;
 #pragma unroll
-        for (int a = 0; a < D; ++a) s += fx_int(up[a], ed) - fx_int(uc[a], ed);
-        val = __ll2double_rn(s) * c;
+        for (int a = 0; a < D; ++a) s += fx_int(up[a], ed) - fx_int(own[a], ed);
+        val[D] = __ll2double_rn(s) * c;
     } else {
         double s = 0.0;
 #pragma unroll
-        for (int a = 0; a < D; ++a) s += up[a] - uc[a];
-        val = -s * ih;
+        for (int a = 0; a < D; ++a) s += (double)up[a] - (double)own[a];
+        val[D] = -s * ih;
     }
-    y[D * g.ncell + n.c] = val;
+}
+
+// y = the product; z (may be NULL): x itself in FP64, written on the way (x is the
+// preconditioner's result, so that no separate conversion reads it)
+template <int D, typename Ti>
+__global__ void __launch_bounds__(256) k_stokes_fx(const Ti* __restrict__ x, double* __restrict__ y,
+                                                   double* __restrict__ z, Geo g, double sigma, double kh2, double ih,
+                                                   const double* __restrict__ shift) {
+    pdl_start();
+    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
+    if (i >= g.n0 || j >= g.n1) return;
+    const Nbr n = neighbours<D>(g, i, j, k);
+    double val[D + 1];
+    Ti own[D + 1];
+    fx_rows<D, Ti>(x, g, n, sigma, kh2, ih, val, own);
+#pragma unroll
+    for (int a = 0; a <= D; ++a) {
+        y[a * g.ncell + n.c] = shift && a < D ? val[a] + shift[a] : val[a];
+        if (z) z[a * g.ncell + n.c] = fx_val(own[a]);
+    }
+}
+
+// ---- the product of an inner step with its dots --------------------------------
+// w = L z (k_stokes' rows) and, in the same sweep, its dots with the basis of the
+// inner solve (V_0 = r, V_1 .. V_NW at Vv, stride ld), with itself, and V_NW's own:
+// the products are read while they are in registers instead of by two more passes
+// and a reduction kernel.  The basis is orthogonal but not normalised (P_S is
+// linear, so the scale of a direction does not matter, and nothing waits for a
+// norm).  The last block to finish sums the blocks' partial sums in a fixed order
+// and enters the column (inner_column).  Blocks of 32 x 8 threads walk tiles of one
+// plane.
+
+// Column j: hs[i * INNER_MAX + j] = h_ij = V_i . w / |V_i|^2, nv[i] = |V_i|^2; y: the h_ij for
+// the next direction w - sum_i h_ij V_i or, after the last column, the y that minimise
+// |V_0 - sum_j y_j L z_j|, from the normal equations of the Hessenberg matrix in the
+// normalised basis.  A direction that adds nothing gets zero.
+__device__ void inner_column(const double* dots, int j, bool fin, double* hs, double* nv, double* y) {
+    nv[j] = dots[j + 2];
+    double rest = dots[j + 1];  // |w|^2 - sum h^2 |V|^2 = |V_{j+1}|^2
+    for (int i = 0; i <= j; ++i) {
+        const double h = nv[i] > 0.0 ? dots[i] / nv[i] : 0.0;
+        hs[i * INNER_MAX + j] = h;
+        rest -= h * dots[i];
+        y[i] = h;
+    }
+    if (!fin) return;
+    double m[INNER_MAX + 1][INNER_MAX], l[INNER_MAX][INNER_MAX], t[INNER_MAX];
+    for (int i = 0; i <= j + 1; ++i) {
+        const double nr = sqrt(i <= j ? nv[i] : fmax(rest, 0.0));
+        for (int q = 0; q <= j; ++q) m[i][q] = i <= q ? hs[i * INNER_MAX + q] * nr : (i == q + 1 ? nr : 0.0);
+    }
+    for (int a = 0; a <= j; ++a) {
+        double d = 0.0;
+        for (int b = 0; b <= a; ++b) {
+            double g = 0.0;
+            for (int i = 0; i <= b + 1; ++i) g += m[i][a] * m[i][b];
+            d = g;
+            for (int q = 0; q < b; ++q) g -= l[a][q] * l[b][q];
+            if (a == b)
+                l[a][a] = g > 1e-14 * d ? 1.0 / sqrt(g) : 0.0;  // the inverse
+            else
+                l[a][b] = g * l[b][b];
+        }
+        double c = m[0][a] * sqrt(nv[0]);
+        for (int q = 0; q < a; ++q) c -= l[a][q] * t[q];
+        t[a] = c * l[a][a];
+    }
+    for (int a = j; a >= 0; --a) {
+        double c = t[a];
+        for (int q = a + 1; q <= j; ++q) c -= l[q][a] * y[q];
+        y[a] = c * l[a][a];
+    }
+}
+
+template <int D, bool W, int NW, typename T>
+__global__ void __launch_bounds__(256) k_stokes_dots(const T* __restrict__ z, T* __restrict__ w, const T* __restrict__ r,
+                                                     const T* __restrict__ Vv, long long ld, Geo g, T sigma, T kh2, T ih,
+                                                     FastDiv dx, FastDiv dy, int ntile, int fin,
+                                                     double* __restrict__ partial, unsigned* __restrict__ ticket,
+                                                     double* __restrict__ hs, double* __restrict__ nv,
+                                                     double* __restrict__ y) {
+    pdl_start();
+    constexpr int NQ = NW + 3;  // V_0 .. V_NW, w, V_NW's own
+    T acc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = T(0);
+    const int mx = (g.n0 + BX - 1) / BX, my = (g.n1 + BY - 1) / BY;
+    auto put = [&](long long e, T val) {
+        if (!fin) w[e] = val;  // the last product itself is not needed
+        T v = r[e];
+        acc[0] += val * v;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            v = Vv[q * ld + e];
+            acc[q + 1] += val * v;
+        }
+        acc[NW + 1] += val * val;
+        acc[NW + 2] += v * v;
+    };
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        const int t = fdiv(tile, dx), k = fdiv(t, dy);
+        const int i = (tile - t * mx) * BX + threadIdx.x, j = (t - k * my) * BY + threadIdx.y;
+        if (i >= g.n0 || j >= g.n1) continue;
+        const Nbr n = neighbours<D>(g, i, j, k);
+        if constexpr (!W && std::is_same<T, double>::value) {
+            double val[D + 1], own[D + 1];
+            fx_rows<D, double>(z, g, n, sigma, kh2, ih, val, own);
+#pragma unroll
+            for (int a = 0; a <= D; ++a) put(a * g.ncell + n.c, val[a]);
+            continue;
+        }
+        const T* p = z + D * g.ncell;
+        const T pc = p[n.c];
+        T div = T(0);
+        const int pm[3] = {n.xm, n.ym, n.zm};
+        const int pp[3] = {n.xp, n.yp, n.zp};
+        const int id[3] = {i, j, k};
+        const int ns[3] = {g.n0, g.n1, g.n2};
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const T* u = z + a * g.ncell;
+            const T uc = u[n.c];
+            T val;
+            if (!W) {
+                const T lap = nbr_sum<D, T>(u, n) - T(2 * D) * uc;
+                val = sigma * uc - kh2 * lap + (pc - p[n.c + pm[a]]) * ih;
+                div += u[n.c + pp[a]] - uc;
+            } else {
+                const WInfo wi = wall_info<D>(g, a, i, j, k);
+                if (wi.ident) {
+                    val = uc;
+                } else {
+                    const T lap = nbr_sum_w<D, T>(u, n, wi.ok) + T(wi.adj - 2 * D) * uc;
+                    val = sigma * uc - kh2 * lap + (pc - p[n.c + pm[a]]) * ih;
+                }
+                const bool wa = (g.wall >> a) & 1;
+                const T hi = (wa && id[a] == ns[a] - 1) ? T(0) : u[n.c + pp[a]];
+                const T lo = (wa && id[a] == 0) ? T(0) : uc;
+                div += hi - lo;
+            }
+            put(a * g.ncell + n.c, val);
+        }
+        put(D * g.ncell + n.c, -div * ih);
+    }
+    // block sums: warps in T, across warps in FP64
+    __shared__ double sm[8][NQ];
+    __shared__ double tot[NQ];
+    __shared__ bool last;
+    const int tid = threadIdx.y * BX + threadIdx.x, lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        T x = acc[q];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) sm[wid][q] = (double)x;
+    }
+    __syncthreads();
+    if (tid < NQ) {
+        double x = 0.0;
+        for (int v = 0; v < 8; ++v) x += sm[v][tid];
+        partial[tid * gridDim.x + blockIdx.x] = x;
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int q = wid; q < NQ; q += 8) {
+        double x = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) x += __ldcg(partial + q * gridDim.x + b);
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) tot[q] = x;
+    }
+    __syncthreads();
+    if (tid == 0) inner_column(tot, NW, fin != 0, hs, nv, y);
 }
 
 // ---- point operators of the per-level kernels (the legs, the tail and the cluster
@@ -1777,6 +1976,17 @@ void wall_set_faces(const Geo& g, int a, const double* data, double* x, cudaStre
     IBR_CHECK_LAUNCH();
 }
 
+template <typename Ti>
+void stokes_apply_from(const Geo& g, const Ti* x, double* y, double* z, double sigma, double eta, const double* shift_dev,
+                       cudaStream_t s) {
+    if (g.wall) throw Error{IBR_EINVAL, "stokes_apply_from: periodic grids only"};
+    const dim3 grid((g.n0 + BX - 1) / BX, (g.n1 + BY - 1) / BY, g.n2), blk(BX, BY);
+    ProfScope ps(KID_STOKES, s, (g.d + 1.0) * g.ncell * (sizeof(Ti) + (z ? 16.0 : 8.0)));
+    launch_k(g.d == 3 ? k_stokes_fx<3, Ti> : k_stokes_fx<2, Ti>, grid, blk, 0, s, x, y, z, g, sigma, eta / (g.h * g.h),
+             1.0 / g.h, shift_dev);
+    IBR_CHECK_LAUNCH();
+}
+
 template <typename T>
 void stokes_apply(const Geo& g, const T* x, T* y, double sigma, double eta, const double* shift_dev,
                   cudaStream_t s) {
@@ -1787,11 +1997,7 @@ void stokes_apply(const Geo& g, const T* x, T* y, double sigma, double eta, cons
     const bool w = g.wall != 0;
     if constexpr (std::is_same<T, double>::value) {
         if (!w) {
-            if (g.d == 3)
-                launch_k(k_stokes_fx<3>, grid, blk, 0, s, x, y, g, sigma, kh2, ih, shift_dev);
-            else
-                launch_k(k_stokes_fx<2>, grid, blk, 0, s, x, y, g, sigma, kh2, ih, shift_dev);
-            IBR_CHECK_LAUNCH();
+            stokes_apply_from<double>(g, x, y, nullptr, sigma, eta, shift_dev, s);
             return;
         }
     }
@@ -1805,6 +2011,36 @@ void stokes_apply(const Geo& g, const T* x, T* y, double sigma, double eta, cons
             launch_k(k_stokes<2, true, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih, shift_dev);
         else
             launch_k(k_stokes<2, false, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih, shift_dev);
+    }
+    IBR_CHECK_LAUNCH();
+}
+
+template <typename T>
+void stokes_dots(const Geo& g, const T* z, T* w, const T* r, const T* Vv, long long ld, int nw, bool fin, double sigma,
+                 double eta, double* partial, unsigned* ticket, double* hs, double* nv, double* y, cudaStream_t s) {
+    const T kh2 = (T)(eta / (g.h * g.h)), ih = (T)(1.0 / g.h), sg = (T)sigma;
+    const int mx = (g.n0 + BX - 1) / BX, my = (g.n1 + BY - 1) / BY, nt = mx * my * g.n2;
+    const dim3 grid(std::min(nt, INNER_BLOCKS)), blk(BX, BY);
+    const FastDiv dx = make_fastdiv(mx), dy = make_fastdiv(my);
+    ProfScope ps(KID_STOKES, s, ((fin ? 2.0 : 3.0) + nw) * (g.d + 1) * g.ncell * sizeof(T));
+    auto go = [&](auto* k) {
+        launch_k(k, grid, blk, 0, s, z, w, r, Vv, ld, g, sg, kh2, ih, dx, dy, nt, fin ? 1 : 0, partial, ticket, hs, nv, y);
+    };
+    auto pick = [&](auto D, auto W) {
+        constexpr int d = decltype(D)::value;
+        constexpr bool wl = decltype(W)::value;
+        if (nw == 0) go(k_stokes_dots<d, wl, 0, T>);
+        else if (nw == 1) go(k_stokes_dots<d, wl, 1, T>);
+        else if (nw == 2) go(k_stokes_dots<d, wl, 2, T>);
+        else go(k_stokes_dots<d, wl, 3, T>);
+    };
+    using I2 = std::integral_constant<int, 2>;
+    using I3 = std::integral_constant<int, 3>;
+    if (nw < 0 || nw >= INNER_MAX) throw Error{IBR_EINVAL, "stokes_dots: at most 3 earlier steps"};
+    if (g.d == 3) {
+        if (g.wall) pick(I3{}, std::true_type{}); else pick(I3{}, std::false_type{});
+    } else {
+        if (g.wall) pick(I2{}, std::true_type{}); else pick(I2{}, std::false_type{});
     }
     IBR_CHECK_LAUNCH();
 }
@@ -2545,6 +2781,8 @@ void wall_lift(const Geo& g, int a, int side, const double* data, double* b, dou
 
 #define IBR_INST(T)                                                                                        \
     template void stokes_apply<T>(const Geo&, const T*, T*, double, double, const double*, cudaStream_t); \
+    template void stokes_dots<T>(const Geo&, const T*, T*, const T*, const T*, long long, int, bool, double, double, \
+                                 double*, unsigned*, double*, double*, double*, cudaStream_t);                 \
     template void mg_smooth<T>(const Geo&, T*, const T*, int, int, double, double, int, bool, cudaStream_t); \
     template void mg_residual_restrict<T>(const Geo&, const Geo&, const T*, const T*, T*, int, int, double, \
                                           double, cudaStream_t);                                          \
@@ -2559,5 +2797,9 @@ void wall_lift(const Geo& g, int a, int side, const double* data, double* b, dou
 IBR_INST(double)
 IBR_INST(float)
 #undef IBR_INST
+template void stokes_apply_from<double>(const Geo&, const double*, double*, double*, double, double, const double*,
+                                        cudaStream_t);
+template void stokes_apply_from<float>(const Geo&, const float*, double*, double*, double, double, const double*,
+                                       cudaStream_t);
 
 }  // namespace ibr
