@@ -260,6 +260,22 @@ __device__ __forceinline__ void pair_window_f(const Geo& g, const double* p, int
     }
 }
 
+// The table keeps the force directions of one cell and velocity component together
+// (PairW floats, one load): the gathers bound this kernel by the sectors they touch
+// in the L2, and separate arrays touch up to three times as many.  With the wrapped
+// offsets formed once per window instead of once per entry: 1307 us for 1184 markers
+// in 3-D against 3145 us before, 96 us for 240 in 2-D.
+template <int D>
+struct PairW;
+template <>
+struct PairW<2> {
+    using type = float2;
+};
+template <>
+struct PairW<3> {
+    using type = float4;
+};
+
 template <int D, int KW>
 __global__ void __launch_bounds__(256) k_pair_mtilde(Geo g, int nr, const double* __restrict__ q, int S,
                                                      const double* __restrict__ x0, const float* __restrict__ tab,
@@ -268,6 +284,7 @@ __global__ void __launch_bounds__(256) k_pair_mtilde(Geo g, int nr, const double
     const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
     if (i >= nr || j >= nr || j < i) return;
     const int ns[3] = {g.n0, g.n1, g.n2};
+    using TW = typename PairW<D>::type;
     // acc[0]: sum_s T_s(q_i - q_j);  acc[1]: sum_s T_s(q_j - q_i)^T
     double acc[2][D][D];
 #pragma unroll
@@ -289,30 +306,52 @@ __global__ void __launch_bounds__(256) k_pair_mtilde(Geo g, int nr, const double
             }
 #pragma unroll
             for (int al = 0; al < D; ++al) {
-                int j0[D];
+                int j0[D], o[D][KW];  // (a table of 2^31 cells would not fit the memory)
                 float w[D][KW];
                 pair_window_f<D, KW>(g, p, al, j0, w);
-                float sum[D];
+                int stride = 1;
 #pragma unroll
-                for (int be = 0; be < D; ++be) sum[be] = 0.0f;
-                const int S_win = D == 3 ? KW * KW * KW : KW * KW;
-                for (int c = 0; c < S_win; ++c) {
-                    long long cell = 0, stride = 1;
-                    float wt = 1.0f;
-                    int cc = c;
+                for (int b = 0; b < D; ++b) {
 #pragma unroll
-                    for (int b = 0; b < D; ++b) {
-                        const int m = cc % KW;
-                        cc /= KW;
-                        int jj = (j0[b] + m) % ns[b];
-                        if (jj < 0) jj += ns[b];
-                        cell += jj * stride;
-                        stride *= ns[b];
-                        wt *= w[b][m];
+                    for (int m = 0; m < KW; ++m) {
+                        int jj = j0[b] + m;
+                        if (jj < 0 || jj >= ns[b]) {
+                            jj %= ns[b];
+                            if (jj < 0) jj += ns[b];
+                        }
+                        o[b][m] = jj * stride;
                     }
+                    stride *= ns[b];
+                }
+                const TW* tb = reinterpret_cast<const TW*>(tab) + (long long)(s * D + al) * g.ncell;
+                float sum[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+                for (int m2 = 0; m2 < (D == 3 ? KW : 1); ++m2) {
 #pragma unroll
-                    for (int be = 0; be < D; ++be)
-                        sum[be] = fmaf(wt, tab[((long long)(s * D + be) * D + al) * g.ncell + cell], sum[be]);
+                    for (int m1 = 0; m1 < KW; ++m1) {
+                        int base = o[1][m1];
+                        float wr = w[1][m1];
+                        if constexpr (D == 3) {
+                            // (m2 is not unrolled: its entry is picked without indexing registers)
+                            int o2 = o[2][0];
+                            float w2 = w[2][0];
+#pragma unroll
+                            for (int e = 1; e < KW; ++e) {
+                                o2 = m2 == e ? o[2][e] : o2;
+                                w2 = m2 == e ? w[2][e] : w2;
+                            }
+                            base += o2;
+                            wr *= w2;
+                        }
+#pragma unroll
+                        for (int m0 = 0; m0 < KW; ++m0) {
+                            const float wt = w[0][m0] * wr;
+                            const TW t = __ldg(tb + base + o[0][m0]);
+                            sum[0] = fmaf(wt, t.x, sum[0]);
+                            sum[1] = fmaf(wt, t.y, sum[1]);
+                            if constexpr (D == 3) sum[2] = fmaf(wt, t.z, sum[2]);
+                        }
+                    }
                 }
 #pragma unroll
                 for (int be = 0; be < D; ++be) {
@@ -334,6 +373,12 @@ __global__ void __launch_bounds__(256) k_pair_mtilde(Geo g, int nr, const double
             M[((long long)i * D + a) * ld + (long long)j * D + b] = v;
             M[((long long)j * D + b) * ld + (long long)i * D + a] = v;  // exactly symmetric
         }
+}
+
+// the velocity x (D components) of one source and force direction into the table
+__global__ void k_pair_store(long long n, int d, int width, const double* __restrict__ x, float* __restrict__ tab) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t < (long long)d * n) tab[t * width] = (float)x[t];
 }
 
 template <int D, int KW>
@@ -438,6 +483,14 @@ void pair_mtilde(const Geo& g, int nr, const double* q, int S, const double* x0,
         else
             k_pair_mtilde<2, 4><<<grid, blk, 0, s>>>(g, nr, q, S, x0, tab, M);
     }
+    IBR_CHECK_LAUNCH();
+}
+
+void pair_store(const Geo& g, int s, int beta, const double* x, float* tab, cudaStream_t st) {
+    const int width = pair_width(g.d);
+    ProfScope ps(KID_CONVERT, st, (double)g.d * g.ncell * 12.0);
+    k_pair_store<<<grid_1d((long long)g.d * g.ncell, 256), 256, 0, st>>>(
+        g.ncell, g.d, width, x, tab + (long long)s * g.d * g.ncell * width + beta);
     IBR_CHECK_LAUNCH();
 }
 

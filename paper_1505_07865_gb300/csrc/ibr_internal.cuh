@@ -550,14 +550,17 @@ void mtilde_build(int d, int Nb, const double* rel_b, const MobParams& p, double
 // set to (k+1) if the k-th pivot is <= min_pivot.  work >= n*n.
 // The pair-mobility table of a periodic grid: for S source points x0[s]
 // and force directions beta, the velocity field v = L^-1 S~ (unit force
-// e_beta at x0[s]) stored in FP32 as tab[((s*d + beta)*d + alpha)*ncell + cell]
-// (alpha: velocity component).  pair_mtilde builds the dense block of the
+// e_beta at x0[s]) stored in FP32 as tab[((s*d + alpha)*ncell + cell)*width + beta]
+// (alpha: velocity component; width: pair_width, the directions padded to a
+// vector load).  pair_store writes one source's and direction's field.  pair_mtilde builds the dense block of the
 // nr markers at positions q[nr][d] (row-major, (d nr)^2):
 //   M~_ij^{ab} = (1/2S) sum_s [ J_a(x0_s + q_i - q_j) v^{s,b} + J_b(x0_s + q_j - q_i) v^{s,a} ]
 // (exactly symmetric).  point_spread writes y[beta*ncell + .] = scale * the
 // 4^d kernel weights of component beta at x0 (periodic; other entries untouched).
 void pair_mtilde(const Geo& g, int nr, const double* q, int S, const double* x0, const float* tab, double* M,
                  cudaStream_t s);
+inline int pair_width(int d) { return d == 3 ? 4 : 2; }
+void pair_store(const Geo& g, int s, int beta, const double* x, float* tab, cudaStream_t st);
 void point_spread(const Geo& g, const double* x0, int beta, double scale, double* y, cudaStream_t s);
 template <typename T>
 void spd_inverse(int n, T* M, T* work, int* info_dev, double min_pivot, cudaStream_t s);

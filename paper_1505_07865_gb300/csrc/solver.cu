@@ -884,7 +884,7 @@ void build_pair_table_into(ibr_grid* G, float*& tab_out, double*& x0_out) {
     double hx0[PAIR_S * 3];
     for (int k = 0; k < PAIR_S; ++k)
         for (int a = 0; a < d; ++a) hx0[k * d + a] = (std::floor(0.5 * G->n[a]) + frac[k][a]) * g.h;
-    float* tab = dalloc<float>((size_t)PAIR_S * d * d * n);
+    float* tab = dalloc<float>((size_t)PAIR_S * d * pair_width(d) * n);
     double* x0 = dalloc<double>((size_t)PAIR_S * d);
     PC<double> pc(G, PAIR_NS);
     double* rhs = dalloc<double>(nS);
@@ -935,7 +935,7 @@ void build_pair_table_into(ibr_grid* G, float*& tab_out, double*& x0_out) {
                     block_means<double>(n, d, x, pc.partial, pc.means, s);
                     subtract_means<double>(n, d, x, pc.means, s);
                 }
-                vec_convert<double, float>((long long)d * n, x, tab + (size_t)(k * d + be) * d * n, s);
+                pair_store(g, k, be, x, tab, s);
             }
         IBR_CUDA_TRY(cudaStreamSynchronize(s));
     } catch (...) {
@@ -1649,7 +1649,7 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
     // preconditioner with PAIR_NS inner vectors and four solve vectors; its
     // blocks: one for all markers while d N <= PAIR_FULL_MAX
     if (mob_model == IBR_MOB_PAIR) {
-        t += pg(4.0 * PAIR_S * d * d * nc);
+        t += pg(4.0 * PAIR_S * d * pair_width(d) * nc);
         double mg64 = 0.0;
         Geo c2 = g;
         while (Multigrid<double>::can_coarsen(c2)) {
