@@ -531,24 +531,25 @@ def run_ours(args, world, rank, local):
                          "share_of_profiled_step": kms / prof_total},
     }
     if kname == "krylov_update_mdot":
-        roof["note"] = ("outer orthogonalisation passes (modified Gram-Schmidt over the FP64 basis, k_mgs_step: V_i, "
-                        "V_{i+1} and w read, w written, two FP64 FMAs per entry); bound by HBM and the FP64 pipe "
-                        "together, see orthogonalisation_roofline for the FP64 fraction")
+        roof["note"] = ("outer orthogonalisation passes (modified Gram-Schmidt over the FP64 basis, k_mgs_block: up to "
+                        "16 basis vectors and w read, w written, two FP64 FMAs per entry and vector); bound by the "
+                        "FP64 pipe, see orthogonalisation_roofline for the FP64 fraction")
     if kname == "mg_smooth_rbgs":
         roof["note"] = ("finest-level half sweeps in red-black split layout (k_rb_first/k_rb_half, 3 stacked fields), "
                         "timed per pre- or post-smoothing sequence of back-to-back launches (two CUDA events per "
                         "sequence, the average over its launches); in the solve the level's u and f (50 MB) stay in "
                         "L2 between half sweeps, so ncu in situ measures almost no DRAM traffic per launch; the HBM "
                         "copy rate is the denominator all the same")
-    # the outer orthogonalisation's passes (modified Gram-Schmidt: V_i, V_{i+1}
-    # and w read, w written; two FP64 FMAs per entry): HBM and FP64 fractions
+    # the outer orthogonalisation's passes (modified Gram-Schmidt: two blocks of
+    # vectors and w read, w written; two FP64 FMAs per entry and vector): HBM and
+    # FP64 fractions
     orth = None
     mg = prof4.get("krylov_update_mdot@large")
     if mg and mg[0] > 0 and os.environ.get("IBR_ARNOLDI", "") in ("", "mgs"):
         gbs = mg[2] / (mg[1] * 1e-3) / 1e9
         tflops = mg[3] / (mg[1] * 1e-3) / 1e12
         fp64_peak = 1.19  # TFLOP/s, measured on this machine's GB300 (FMA-throughput probe)
-        orth = {"kernel": "k_mgs_step", "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
+        orth = {"kernel": "k_mgs_block", "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
                 "frac": gbs / hbm, "fp64_tflops": tflops, "fp64_frac": tflops / fp64_peak,
                 "avg_launch_us": mg[1] / mg[0] * 1000.0, "launches_per_step": mg[0] / args.profile_steps,
                 "algorithmic_bytes_per_launch": mg[2] / mg[0]}

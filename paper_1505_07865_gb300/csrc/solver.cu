@@ -1,9 +1,9 @@
 // Host orchestration and the C ABI of libibrigid.
 //
 // Outer solver: right-preconditioned flexible GMRES in FP64 on the
-// constrained system (Sec. V), Arnoldi by classical Gram-Schmidt with a
-// second pass only when needed, Givens rotations on the device, true residual
-// recomputed at every restart and at exit.
+// constrained system (Sec. V), Arnoldi by modified Gram-Schmidt in blocks of
+// eight vectors, Givens rotations on the device, true residual recomputed at
+// every restart and at exit.
 // Preconditioner: the Schur-complement preconditioner of Sec. V.A
 //   1. inner GMRES(N_s) on the unconstrained Stokes system, each step
 //      preconditioned by P_S (Sec. V.B, Eq. P1_practical) = one vector
