@@ -1027,7 +1027,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
     k_mgs_block(long long n2, long long ld2, const double2* __restrict__ Vs, const double2* __restrict__ Vd,
                 double2* __restrict__ w, const double* __restrict__ L, const double* __restrict__ pin,
                 double* __restrict__ pout, double* __restrict__ hcol) {
-    pdl_start();
+    pdl_start(Vs, Vd, w, L, pin);
     constexpr bool LAST = ND == 0, GRAM = LAST && NS < MGS_B;
     constexpr int NQ = LAST ? NS + 1 : ND;
     __shared__ double buf[NQ * RED_THREADS];
@@ -1059,6 +1059,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
         double2 v[NS > 0 ? NS : 1], d[ND > 0 ? ND : 1];
 #pragma unroll
         for (int q = 0; q < NS; ++q) v[q] = __ldcs(Vs + q * ld2 + p);
+        // (read-only path: no kernel that may still run as this one starts writes basis vectors)
 #pragma unroll
         for (int q = 0; q < ND; ++q) d[q] = __ldg(Vd + q * ld2 + p);
 #pragma unroll
@@ -1142,7 +1143,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_norm(long long n2, const do
                                                           const double* __restrict__ h, int j, double* cs, double* sn,
                                                           double* gv, double* res_out, double* __restrict__ out64,
                                                           long long from64, long long n64) {
-    pdl_start();
+    pdl_start(w, pin);
     __shared__ double sums[MGS_B + 1];
     __shared__ double piece[2];
     __shared__ double sm[3 * 128];
@@ -1186,6 +1187,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_norm(long long n2, const do
             if (out32 && i < n32) out32[i] = (float)x.x;
             if (out32 && i + 1 < n32) out32[i + 1] = (float)x.y;
         }
+        pdl_behind(h, cs, sn, gv);
         if (ng > 0) {
             mgs_collect(pin, nblk, ng, sums);
             if (threadIdx.x < ng) grow[threadIdx.x] = sums[threadIdx.x] * inv;
@@ -1453,10 +1455,10 @@ template <int K, typename T>
 __global__ void __launch_bounds__(256) k_inner_direction(long long n, T* __restrict__ w, const T* __restrict__ r,
                                                          const T* __restrict__ V, long long ld,
                                                          const double* __restrict__ y, int vec) {
-    pdl_start();
+    pdl_start(w, r, V, y);
     T c[K];
 #pragma unroll
-    for (int i = 0; i < K; ++i) c[i] = (T)pdl_ld(y + i);
+    for (int i = 0; i < K; ++i) c[i] = (T)y[i];
     const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (vec) {
         for (long long q = t0; q < n / 4; q += stride) {
@@ -1485,10 +1487,10 @@ __global__ void __launch_bounds__(256) k_inner_combine(long long m, const T* __r
                                                        const double* __restrict__ y, T* __restrict__ x, int d,
                                                        double* __restrict__ means, double* __restrict__ partial,
                                                        unsigned* __restrict__ ticket, int vec) {
-    pdl_start();
+    pdl_start(Z, y);
     T c[K];
 #pragma unroll
-    for (int i = 0; i < K; ++i) c[i] = (T)pdl_ld(y + i);
+    for (int i = 0; i < K; ++i) c[i] = (T)y[i];
     const int cmp = blockIdx.y;
     Z += (long long)cmp * m;
     x += (long long)cmp * m;
@@ -1535,6 +1537,7 @@ __global__ void __launch_bounds__(256) k_inner_combine(long long m, const T* __r
     }
     __syncthreads();
     if (!last || threadIdx.x >= 32) return;
+    pdl_behind(partial);
     __threadfence();
     double t = 0.0;
     for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) t += __ldcg(partial + cmp * gridDim.x + b);

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(128) k_spread_interp(Geo g, int N, int nsb, lo
                                                        const double* __restrict__ w, const double* __restrict__ v,
                                                        double* __restrict__ out, double sign,
                                                        const double* __restrict__ mean) {
-    pdl_start();
+    pdl_start(face, off, ent_m, ew, lam, y, idx, w, v, mean);
     if ((int)blockIdx.x < nsb) {
         const long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x;
         if (f >= F) return;

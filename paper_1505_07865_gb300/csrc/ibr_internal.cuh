@@ -93,18 +93,36 @@ bool profiling_enabled();
 // while its predecessor drains (its launch latency overlaps the predecessor's
 // last wave); it lets its own successor do the same (pdl_start) and waits for
 // the predecessor's results in hardware (griddepcontrol.wait) before reading
-// any input.  Kernels launched this way call pdl_start() first; outside a
-// programmatic launch both are no-ops.  IBR_PDL=0 in the environment: plain
+// any input.  Kernels launched this way call pdl_start(pointers) first; outside a
+// programmatic launch it does nothing.  IBR_PDL=0 in the environment: plain
 // launches.
-__device__ __forceinline__ void pdl_start() {
+//
+// The wait alone does not order a kernel's loads: the compiler may take what a
+// const __restrict__ parameter points to as unchanged for the kernel's whole life,
+// load it through the read-only path and schedule that load ahead of the wait (seen
+// where no branch lay between them).  So every pointer that a kernel reads is passed
+// to pdl_start (or, where only a late part of the kernel reads it and registers are
+// short, to pdl_behind there): it comes back as a value that an empty volatile asm
+// statement after the wait has produced, of which the compiler knows nothing but
+// its address space.  A load through it depends on that statement, and it is
+// a plain ld.global, which the wait orders.
+template <typename P>
+__device__ __forceinline__ void pdl_hide(P& p) {
+    size_t a = __cvta_generic_to_global(p);
+    asm volatile("" : "+l"(a));
+    p = static_cast<P>(__cvta_global_to_generic(a));
+}
+template <typename... P>
+__device__ __forceinline__ void pdl_behind(P&... p) {
+    (pdl_hide(p), ...);
+}
+template <typename... P>
+__device__ __forceinline__ void pdl_start(P&... p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_behind(p...);
 }
 bool pdl_enabled();
-// A value that the predecessor wrote, read at the very start of a kernel: through a
-// const __restrict__ pointer such a load may be scheduled ahead of the wait in
-// pdl_start when no branch lies between them; a volatile one is not.
-__device__ __forceinline__ double pdl_ld(const double* p) { return *reinterpret_cast<const volatile double*>(p); }
 
 // Bulk asynchronous copies into shared memory with completion counted on an
 // mbarrier (the producer / consumer pipelines of the tensor-core products and

@@ -159,13 +159,13 @@ constexpr int BX = 32, BY = 8;
 template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_stokes(const T* __restrict__ x, T* __restrict__ y, Geo g, T sigma, T kh2,
                                                 T ih, const double* __restrict__ shift) {
-    pdl_start();
+    pdl_start(x, shift);
     int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
     if (i >= g.n0 || j >= g.n1) return;
     Nbr n = neighbours<D>(g, i, j, k);
     const T* p = x + D * g.ncell;
     T pc = p[n.c];
-    T div = T(0);
+    T div = T(0), rows[D + 1];
     const int pm[3] = {n.xm, n.ym, n.zm};
     const int pp[3] = {n.xp, n.yp, n.zp};
     const int id[3] = {i, j, k};
@@ -193,9 +193,11 @@ __global__ void __launch_bounds__(256) k_stokes(const T* __restrict__ x, T* __re
             div += hi - lo;
         }
         if (shift) val += (T)shift[a];
-        y[a * g.ncell + n.c] = val;
+        rows[a] = val;
     }
-    y[D * g.ncell + n.c] = -div * ih;
+    rows[D] = -div * ih;
+#pragma unroll
+    for (int a = 0; a <= D; ++a) y[a * g.ncell + n.c] = rows[a];
 }
 
 // ---- the same product with the sums in 64-bit integers (periodic grids, FP64) ----
@@ -319,7 +321,7 @@ template <int D, typename Ti>
 __global__ void __launch_bounds__(256) k_stokes_fx(const Ti* __restrict__ x, double* __restrict__ y,
                                                    double* __restrict__ z, Geo g, double sigma, double kh2, double ih,
                                                    const double* __restrict__ shift) {
-    pdl_start();
+    pdl_start(x, shift);
     const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
     if (i >= g.n0 || j >= g.n1) return;
     const Nbr n = neighbours<D>(g, i, j, k);
@@ -341,7 +343,11 @@ __global__ void __launch_bounds__(256) k_stokes_fx(const Ti* __restrict__ x, dou
 // linear, so the scale of a direction does not matter, and nothing waits for a
 // norm).  The last block to finish sums the blocks' partial sums in a fixed order
 // and enters the column (inner_column).  Blocks of 32 x 8 threads walk tiles of one
-// plane.
+// plane.  Bound by memory: a cell's loads all come ahead of its stores, which no
+// plain load may overtake, what is read once is marked so, and the first two FP32
+// steps keep 2048 threads on an SM (192^3, all products of a solve: 162 us each; 170
+// with 40 registers and stores among the loads, 162 with loads through the
+// read-only path, which data of a kernel that may still be running forbids).
 
 // Column j: hs[i * INNER_MAX + j] = h_ij = V_i . w / |V_i|^2, nv[i] = |V_i|^2; y: the h_ij for
 // the next direction w - sum_i h_ij V_i or, after the last column, the y that minimise
@@ -386,29 +392,33 @@ __device__ void inner_column(const double* dots, int j, bool fin, double* hs, do
 }
 
 template <int D, bool W, int NW, typename T>
-__global__ void __launch_bounds__(256) k_stokes_dots(const T* __restrict__ z, T* __restrict__ w, const T* __restrict__ r,
-                                                     const T* __restrict__ Vv, long long ld, Geo g, T sigma, T kh2, T ih,
-                                                     FastDiv dx, FastDiv dy, int ntile, int fin,
-                                                     double* __restrict__ partial, unsigned* __restrict__ ticket,
-                                                     double* __restrict__ hs, double* __restrict__ nv,
-                                                     double* __restrict__ y) {
-    pdl_start();
+__global__ void __launch_bounds__(256, sizeof(T) == 4 && !W && NW < 2 ? 8 : 0)
+    k_stokes_dots(const T* __restrict__ z, T* __restrict__ w, const T* __restrict__ r, const T* __restrict__ Vv,
+                  long long ld, Geo g, T sigma, T kh2, T ih, FastDiv dx, FastDiv dy, int ntile, int fin,
+                  double* __restrict__ partial, unsigned* __restrict__ ticket, double* __restrict__ hs,
+                  double* __restrict__ nv, double* __restrict__ y) {
+    pdl_start(z, r, Vv);
     constexpr int NQ = NW + 3;  // V_0 .. V_NW, w, V_NW's own
     T acc[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = T(0);
     const int mx = (g.n0 + BX - 1) / BX, my = (g.n1 + BY - 1) / BY;
-    auto put = [&](long long e, T val) {
-        if (!fin) w[e] = val;  // the last product itself is not needed
-        T v = r[e];
+    auto dot = [&](long long e, T val) {
+        T v = __ldcs(r + e);
         acc[0] += val * v;
 #pragma unroll
         for (int q = 0; q < NW; ++q) {
-            v = Vv[q * ld + e];
+            v = __ldcs(Vv + q * ld + e);
             acc[q + 1] += val * v;
         }
         acc[NW + 1] += val * val;
         acc[NW + 2] += v * v;
+    };
+    // a cell's rows are stored together: no load of it has to wait behind a store
+    auto put = [&](long long c, const T (&val)[D + 1]) {
+        if (fin) return;  // the last product itself is not needed
+#pragma unroll
+        for (int a = 0; a <= D; ++a) __stcs(w + a * g.ncell + c, val[a]);
     };
     for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
         const int t = fdiv(tile, dx), k = fdiv(t, dy);
@@ -419,12 +429,13 @@ __global__ void __launch_bounds__(256) k_stokes_dots(const T* __restrict__ z, T*
             double val[D + 1], own[D + 1];
             fx_rows<D, double>(z, g, n, sigma, kh2, ih, val, own);
 #pragma unroll
-            for (int a = 0; a <= D; ++a) put(a * g.ncell + n.c, val[a]);
+            for (int a = 0; a <= D; ++a) dot(a * g.ncell + n.c, val[a]);
+            put(n.c, val);
             continue;
         }
         const T* p = z + D * g.ncell;
         const T pc = p[n.c];
-        T div = T(0);
+        T div = T(0), rows[D + 1];
         const int pm[3] = {n.xm, n.ym, n.zm};
         const int pp[3] = {n.xp, n.yp, n.zp};
         const int id[3] = {i, j, k};
@@ -451,9 +462,12 @@ __global__ void __launch_bounds__(256) k_stokes_dots(const T* __restrict__ z, T*
                 const T lo = (wa && id[a] == 0) ? T(0) : uc;
                 div += hi - lo;
             }
-            put(a * g.ncell + n.c, val);
+            rows[a] = val;
+            dot(a * g.ncell + n.c, val);
         }
-        put(D * g.ncell + n.c, -div * ih);
+        rows[D] = -div * ih;
+        dot(D * g.ncell + n.c, rows[D]);
+        put(n.c, rows);
     }
     // block sums: warps in T, across warps in FP64
     __shared__ double sm[8][NQ];
@@ -477,6 +491,7 @@ __global__ void __launch_bounds__(256) k_stokes_dots(const T* __restrict__ z, T*
     if (tid == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
+    pdl_behind(partial, hs, nv, y);
     __threadfence();
     for (int q = wid; q < NQ; q += 8) {
         double x = 0.0;
@@ -672,7 +687,7 @@ __device__ __forceinline__ T prolong_cell(const T* cc, const Geo& gc, int fld, i
 template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_rbgs(T* __restrict__ u, const T* __restrict__ f, Geo g, int fld0, T sigma,
                                               T kh2, T inv_diag, int color, int zero_init) {
-    pdl_start();
+    pdl_start(u, f);
     int ih = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
     int k = blockIdx.z % g.n2, cmp = blockIdx.z / g.n2;
     if (ih >= (g.n0 >> 1) || j >= g.n1) return;
@@ -690,7 +705,7 @@ __global__ void __launch_bounds__(256) k_rbgs(T* __restrict__ u, const T* __rest
 template <typename T>
 __global__ void __launch_bounds__(256) k_rbgs_col(T* __restrict__ u, const T* __restrict__ f, Geo g, int nkb, int kz,
                                                   T kh2, T inv_diag, int color, int zero_init) {
-    pdl_start();
+    pdl_start(u, f);
     const int ih = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     const int cmp = blockIdx.z / nkb, kb = blockIdx.z - cmp * nkb;
     if (ih >= (g.n0 >> 1) || j >= g.n1) return;
@@ -723,7 +738,7 @@ template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_resid_restrict(const T* __restrict__ u, const T* __restrict__ f,
                                                         T* __restrict__ fc, Geo gf, Geo gc, int fld0, T sigma,
                                                         T kh2) {
-    pdl_start();
+    pdl_start(u, f);
     int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y;
     int K = blockIdx.z % gc.n2, cmp = blockIdx.z / gc.n2;
     if (I >= gc.n0 || J >= gc.n1) return;
@@ -735,7 +750,7 @@ __global__ void __launch_bounds__(256) k_resid_restrict(const T* __restrict__ u,
 template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_prolong(T* __restrict__ u, const T* __restrict__ uc, Geo gf, Geo gc,
                                                  int fld0) {
-    pdl_start();
+    pdl_start(u, uc);
     int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
     int k = blockIdx.z % gf.n2, cmp = blockIdx.z / gf.n2;
     if (i >= gf.n0 || j >= gf.n1) return;
@@ -1130,7 +1145,8 @@ __global__ void __launch_bounds__(1024) k_mg_tail(const __grid_constant__ TailLe
                                                   const T* __restrict__ fg,
                                                   int fld0, T sigma, int zero_start, int pre, int post,
                                                   int sweeps) {
-    pdl_start();
+    const T* ur = ug;  // what is read of ug (its stores need no wait of their own)
+    pdl_start(ur, fg);
     extern __shared__ unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
     __shared__ double red[32];
@@ -1139,6 +1155,7 @@ __global__ void __launch_bounds__(1024) k_mg_tail(const __grid_constant__ TailLe
     const int fld = field_of(fld0, cmp);
     const int n0 = (int)tl.g[0].ncell;
     ug += (long long)cmp * n0;
+    ur += (long long)cmp * n0;
     fg += (long long)cmp * n0;
     {
         T* u0 = sm + tl.uoff[0];
@@ -1147,8 +1164,8 @@ __global__ void __launch_bounds__(1024) k_mg_tail(const __grid_constant__ TailLe
         if (!zero_start)
             for (int t = tid; t < (n0 >> 1); t += nt) {
                 const TailPair<D> p = tail_pair<D>(tl, 0, t);
-                u0[p.b * (n0 >> 1) + t] = ug[2 * t];
-                u0[(1 - p.b) * (n0 >> 1) + t] = ug[2 * t + 1];
+                u0[p.b * (n0 >> 1) + t] = ur[2 * t];
+                u0[(1 - p.b) * (n0 >> 1) + t] = ur[2 * t + 1];
             }
     }
     __syncthreads();
@@ -1222,7 +1239,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_rb_first(const T* __restrict__ fnat, T* __restrict__ fs, T* __restrict__ us,
                                                   int n0, int n1, int n2, int nthreads, FastDiv dq, FastDiv d1,
                                                   FastDiv d2, T inv) {
-    pdl_start();
+    pdl_start(fnat);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nthreads) return;
     const int hn = n0 >> 1, hq = hn / RB_V;
@@ -1255,14 +1272,15 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_rb_half(T* __restrict__ us, const T* __restrict__ fs, int n0, int n1, int n2,
                                                  int nthreads, FastDiv dq, FastDiv d1, FastDiv d2, T kh2, T inv,
                                                  int color, T* __restrict__ unat) {
-    pdl_start();
+    const T* ur = us;
+    pdl_start(ur, fs);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nthreads) return;
     const int hn = n0 >> 1, hq = hn / RB_V;
     const RbIdx r = rb_index(t, hq, dq, n1, d1, n2, d2);
     const long long half = (long long)hn * n1 * n2;
     T* dst = us + (long long)(2 * r.q + color) * half;
-    const T* src = us + (long long)(2 * r.q + 1 - color) * half;
+    const T* src = ur + (long long)(2 * r.q + 1 - color) * half;
     const T* f = fs + (long long)(2 * r.q + color) * half;
     const int p = (r.j + r.k + color) & 1;
     const long long plane = (long long)hn * n1;
@@ -1326,7 +1344,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_rb_restrict(const T* __restrict__ us, const T* __restrict__ fs,
                                                      T* __restrict__ fc, int n0, int n1, int n2, int C, T sigma,
                                                      T kh2, FastDiv dc0, FastDiv dc1, FastDiv dc2) {
-    pdl_start();
+    pdl_start(us, fs);
     const int nc0 = n0 >> 1, nc1 = n1 >> 1, nc2 = n2 >> 1;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int ncc = nc0 * nc1 * nc2;
@@ -1373,7 +1391,7 @@ __global__ void __launch_bounds__(256) k_rb_restrict(const T* __restrict__ us, c
 template <typename T>
 __global__ void __launch_bounds__(256) k_rb_prolong(T* __restrict__ us, const T* __restrict__ uc, int n0, int n1,
                                                     int n2, int nthreads, FastDiv dq, FastDiv d1, FastDiv d2) {
-    pdl_start();
+    pdl_start(us, uc);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nthreads) return;
     const int hn = n0 >> 1, hq = hn / RB_V;
@@ -1443,7 +1461,8 @@ template <typename T>
 __global__ void __launch_bounds__(1024) k_mg_cluster(const __grid_constant__ ClusterLevels cl, T* __restrict__ ug,
                                                      const T* __restrict__ fg,
                                                      T sigma, int zero_start, int pre, int post, int sweeps) {
-    pdl_start();
+    const T* ur = ug;
+    pdl_start(ur, fg);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
     __shared__ double red[32];
@@ -1454,6 +1473,7 @@ __global__ void __launch_bounds__(1024) k_mg_cluster(const __grid_constant__ Clu
     const int plane0 = cl.n0[0] * cl.n1[0];
     const long long ncell0 = (long long)plane0 * cl.n2[0];
     ug += cmp * ncell0;
+    ur += cmp * ncell0;
     fg += cmp * ncell0;
     T* tailbase = sm + cl.toff;
 
@@ -1585,7 +1605,7 @@ __global__ void __launch_bounds__(1024) k_mg_cluster(const __grid_constant__ Clu
     {
         T* u0 = sm + cl.uoff[0];
         const int n = cl.P[0] * plane0;
-        const T* src = ug + (long long)r * n;
+        const T* src = ur + (long long)r * n;
         for (int c = tid; c < n; c += nt) u0[c] = zero_start ? T(0) : src[c];
     }
     cluster.sync();
@@ -1756,7 +1776,7 @@ template <bool W, typename T>
 __global__ void __launch_bounds__(1024) k_leg_down(const __grid_constant__ LegArgs a, const T* __restrict__ uin,
                                                    const T* __restrict__ f, T* __restrict__ uout, T* __restrict__ fc,
                                                    T sigma, T kh2, T inv, int pre) {
-    pdl_start();
+    pdl_start(uin, f);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* su = reinterpret_cast<T*>(smem_raw);  // u per colour, then the residual
     const int np = a.hn * a.R1;
@@ -1827,7 +1847,7 @@ template <bool W, typename T>
 __global__ void __launch_bounds__(1024) k_leg_up(const __grid_constant__ LegArgs a, const T* __restrict__ uin,
                                                  const T* __restrict__ uc, const T* __restrict__ f,
                                                  T* __restrict__ uout, T sigma, T kh2, T inv, int post) {
-    pdl_start();
+    pdl_start(uin, uc, f);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* su = reinterpret_cast<T*>(smem_raw);
     const int by = fdiv(blockIdx.x, a.dm0), bx = (int)blockIdx.x - by * a.m0, cmp = blockIdx.y;
@@ -1858,7 +1878,7 @@ __global__ void __launch_bounds__(1024) k_leg_up(const __grid_constant__ LegArgs
 template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_ps_div(const T* __restrict__ y, const T* __restrict__ hd,
                                                 T* __restrict__ qr, T rhs_scale, T* __restrict__ q, Geo g, T ih) {
-    pdl_start();
+    pdl_start(y, hd);
     int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
     if (i >= g.n0 || j >= g.n1) return;
     Nbr n = neighbours<D>(g, i, j, k);
@@ -1889,21 +1909,22 @@ template <int D, bool W, typename T>
 __global__ void __launch_bounds__(256) k_ps_finish(const T* __restrict__ y, const T* __restrict__ phi,
                                                    const T* __restrict__ q, T* __restrict__ z, Geo g, T h, T c_q,
                                                    T c_phi) {
-    pdl_start();
+    pdl_start(y, phi, q);
     int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
     if (i >= g.n0 || j >= g.n1) return;
     Nbr n = neighbours<D>(g, i, j, k);
     const int pm[3] = {n.xm, n.ym, n.zm};
     const int id[3] = {i, j, k};
     T pc = phi[n.c];
+    T val[D + 1];  // (every load ahead of the first store, which may not overtake it: 192^3 74 -> 48 us)
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        if (W && ((g.wall >> a) & 1) && id[a] == 0)
-            z[a * g.ncell + n.c] = y[a * g.ncell + n.c];
-        else
-            z[a * g.ncell + n.c] = y[a * g.ncell + n.c] + h * (pc - phi[n.c + pm[a]]);
+        val[a] = y[a * g.ncell + n.c];
+        if (!(W && ((g.wall >> a) & 1) && id[a] == 0)) val[a] += h * (pc - phi[n.c + pm[a]]);
     }
-    z[D * g.ncell + n.c] = c_q * q[n.c] + c_phi * pc;
+    val[D] = c_q * q[n.c] + c_phi * pc;
+#pragma unroll
+    for (int a = 0; a <= D; ++a) z[a * g.ncell + n.c] = val[a];
 }
 
 // boundary data of one wall into the right-hand side (one thread per face point)
