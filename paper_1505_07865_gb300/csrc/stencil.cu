@@ -232,12 +232,13 @@ __device__ __forceinline__ long long fx_int(float v, int emax) {
     const long long sg = (long long)((int)b >> 31);
     return ((long long)(m >> sh) ^ sg) - sg;
 }
-// c times what one unit of fx_int(., emax) is worth; ok: it is a normal number and the
-// sum's values are far enough from the ends of their type's range
+// c times what one unit of fx_int(., emax) is worth; ok: c and the result are normal
+// numbers (only then does adding to the exponent multiply) and the sum's values are far
+// enough from the ends of their type's range
 __device__ __forceinline__ double fx_times(double c, int q, bool& ok) {
     const int hi = __double2hiint(c);
-    const int e = ((hi >> 20) & 0x7ff) + q;
-    ok = ok && e >= 1 && e < 0x7ff;
+    const int ec = (hi >> 20) & 0x7ff, e = ec + q;
+    ok = ok && ec >= 1 && ec < 0x7ff && e >= 1 && e < 0x7ff;
     return __hiloint2double((hi & 0x800fffff) | (e << 20), __double2loint(c));
 }
 template <typename Ti>

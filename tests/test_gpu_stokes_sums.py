@@ -103,3 +103,23 @@ def test_non_finite_values_reach_the_rows_that_use_them(value):
         want[1, 7 + dz, 6 + dy, 5 + dx] = True
     want[3, 7, 6, 5] = want[3, 7, 5, 5] = True  # the two cells that share the face
     assert np.array_equal(bad, want)
+
+
+def test_an_infinite_coefficient_stays_infinite():
+    """eta h^-2 = 1e310 overflows: no row of it may come out as a number (the scale of the
+    integer sums is formed by adding exponents, which means something for normal numbers only)"""
+    from paper_1505_07865_gb300 import abi
+
+    n, h = 34, 1e-10
+    G = abi.create_grid(2, (n, n), (n * h, n * h), eta=1e290, precision=abi.FP64)
+    try:
+        bid = abi.add_body(G, [0.5 * n * h] * 2)
+        abi.set_markers(G, bid, np.array([[2.0 * h, 0.0], [-2.0 * h, 0.0]]))
+        abi.prepare(G)
+        xt = torch.zeros(abi.sizes(G)[0], dtype=torch.float64, device="cuda")
+        xt[:2 * n * n] = torch.as_tensor(np.random.default_rng(9).standard_normal(2 * n * n), device="cuda")
+        y = torch.empty_like(xt)
+        abi.apply_system(G, xt, y)
+        assert not torch.isfinite(y[:2 * n * n]).any()
+    finally:
+        abi.destroy_grid(G)
