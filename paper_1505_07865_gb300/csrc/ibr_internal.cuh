@@ -316,8 +316,19 @@ template <typename T>
 void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, int C, int fld0, double sigma,
                double kappa, bool zero_start, int pre, int post, int coarse_sweeps, cudaStream_t s,
                T* rb_u = nullptr, T* rb_f = nullptr, T* rb_u1 = nullptr, T* rb_f1 = nullptr, T* const* Wt = nullptr);
-// levels that may run each leg in one launch (and need a temporary for it)
-inline bool mg_leg_level(const Geo& g) { return g.d == 2; }
+// Levels that run each leg in one launch (and need a temporary for it): 2-D ones of at
+// most so many cells, C stacked fields together.  A leg forms the cells of its
+// halo again, 2.3 times the tile's own: a price per cell, while what it saves, the
+// launches of the half sweeps and what they read again, is the same at every size
+// where launches bound them.  FP64 sweeps pay for every cell (two operations per
+// clock and SM), FP32 ones between walls for the boundary rules; on periodic
+// grids FP32 legs stay ahead to 4096^2 (P_S 1657 us, 2345 per half sweep).  The finest
+// level's own share of P_S, legs / half sweeps in us: FP64 512^2 80 / 104, 640^2
+// 151 / 122, 1024^2 380 / 249; FP64 with walls 384^2 88 / 133, 512^2 152 / 154, 640^2
+// 227 / 182; FP32 with walls 768^2 96 / 103, 1024^2 160 / 152, 2048^2 620 / 493.
+inline bool mg_leg_level(const Geo& g, int C, size_t element) {
+    return g.d == 2 && (element == 8 ? C * g.ncell <= 450000 : !g.wall || C * g.ncell <= 1250000);
+}
 // red-black sweeps of the coarsest-level solve: enough for a preconditioner
 // (the coarsest grid has at most a few hundred cells)
 inline int mg_coarse_sweeps(const Geo& g) {

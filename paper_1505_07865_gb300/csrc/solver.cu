@@ -100,7 +100,7 @@ struct Multigrid {
             g = c;
         }
         coarse_sweeps = mg_coarse_sweeps(lev.back());
-        for (const Geo& l : lev) tmp.push_back(mg_leg_level(l) ? dalloc<T>((size_t)cmax * l.ncell) : nullptr);
+        for (const Geo& l : lev) tmp.push_back(mg_leg_level(l, 1, sizeof(T)) ? dalloc<T>((size_t)cmax * l.ncell) : nullptr);
         if (g0.d == 3 && !g0.wall && g0.n0 % 8 == 0 && lev.size() > 1) {
             rb_u = dalloc<T>((size_t)cmax * g0.ncell);
             rb_f = dalloc<T>((size_t)cmax * g0.ncell);
@@ -1625,15 +1625,14 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
     t += pg(e * (ns + 1) * nS) + pg(e * ns * nS) + 4 * pg(e * nS) + pg(e * d * nc) + 3 * pg(e * nc);
     t += pg(8.0 * RED_BLOCKS * std::max(ns + 1, 4)) + 2 * pg(e * dN) + pg(8.0 * dN);
     // the temporaries of the one-launch legs (2-D)
-    Geo lg = g;
-    for (;;) {
-        if (mg_leg_level(lg)) t += pg(e * d * (double)lg.ncell);
-        if (!Multigrid<float>::can_coarsen(lg)) break;
-        lg.n0 /= 2;
-        lg.n1 /= 2;
-        if (d == 3) lg.n2 /= 2;
-        lg.ncell = (long long)lg.n0 * lg.n1 * lg.n2;
-    }
+    auto leg_bytes = [&](double size) {
+        double bytes = 0.0;
+        for (Geo l = g;; l.n0 /= 2, l.n1 /= 2, l.ncell /= 4) {
+            if (mg_leg_level(l, 1, (size_t)size)) bytes += pg(size * d * (double)l.ncell);
+            if (d != 2 || !Multigrid<float>::can_coarsen(l)) return bytes;
+        }
+    };
+    t += leg_bytes(e);
     // the red-black split copies of u and f of the finest level and level 1 (periodic 3-D)
     if (d == 3 && g.n0 % 8 == 0) t += 2 * pg(e * d * nc);
     if (d == 3 && g.n0 % 16 == 0 && Multigrid<float>::can_coarsen(g)) t += 2 * pg(e * d * nc / 8);
@@ -1659,8 +1658,7 @@ long long estimate_grid_bytes(int d, const int* n, int B, const int* Nb, int res
             c2.ncell = (long long)c2.n0 * c2.n1 * c2.n2;
             mg64 += 2 * pg(8.0 * d * (double)c2.ncell);
         }
-        if (mg_leg_level(g)) mg64 += 4.0 / 3.0 * 8.0 * d * nc + 8 * pg(2097152.0);
-        t += mg64 + pg(8.0 * (PAIR_NS + 1) * nS) + pg(8.0 * PAIR_NS * nS) + 8 * pg(8.0 * nS) + pg(8.0 * d * nc) +
+        t += mg64 + leg_bytes(8.0) + pg(8.0 * (PAIR_NS + 1) * nS) + pg(8.0 * PAIR_NS * nS) + 8 * pg(8.0 * nS) + pg(8.0 * d * nc) +
              3 * pg(8.0 * nc);
         if (dN <= (double)pair_full_max()) blk2 = blkmax = dN * dN;
     }

@@ -2470,8 +2470,9 @@ inline dim3 leg_grid(const LegArgs& a, int C) {
 inline int leg_block(const LegArgs& a) { return (a.hn * a.R1 + 31) / 32 * 32; }
 
 // whether a level runs its legs in one launch each
-inline bool leg_ok(const Geo& g, int pre, int post) {
-    return mg_leg_level(g) && pre >= 1 && post >= 1 && pre <= 3 && post <= 3 && g.n0 >= 8 && g.n1 >= 8;
+template <typename T>
+bool leg_ok(const Geo& g, int C, int pre, int post) {
+    return mg_leg_level(g, C, sizeof(T)) && pre >= 1 && post >= 1 && pre <= 3 && post <= 3 && g.n0 >= 8 && g.n1 >= 8;
 }
 template <typename T>
 bool leg_aligned(const T* a, const T* b, const T* c) {
@@ -2515,12 +2516,11 @@ void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, in
     for (int l = 0; l < 2; ++l)
         split_l[l] = L > l + 1 && (long long)C * lev[l].ncell < (1LL << 31) &&
                      rb_split_ok<T>(lev[l], Fl(l), U[l], rbu[l], rbf[l], l > 0 || zero_start, pre, post);
-    // a level runs as two legs where it is small enough for launch latency to
-    // bound it (a level in split layout never is, unless legs take it)
+    // levels that run as two legs (3-D ones, the split layout's among them, never do)
     auto legs = [&](int l) {
-        return Wt && Wt[l] && l + 1 < L && leg_ok(lev[l], pre, post) && leg_aligned<T>(Fl(l), U[l], Wt[l]);
+        return Wt && Wt[l] && l + 1 < L && leg_ok<T>(lev[l], C, pre, post) && leg_aligned<T>(Fl(l), U[l], Wt[l]);
     };
-    auto split = [&](int l) { return l < 2 && split_l[l] && !legs(l); };
+    auto split = [&](int l) { return l < 2 && split_l[l]; };
     // periodic 3-D: the coarse levels on one thread-block cluster per field
     ClusterLevels cl;
     int top = 0;
