@@ -68,47 +68,10 @@ __global__ void k_axpby(long long n, T a, const T* __restrict__ x, T b, T* __res
         y[i] = a * x[i] + b * y[i];
 }
 
-template <typename T>
-__global__ void k_scale_copy(long long n, const double* __restrict__ sc, int invert, const T* __restrict__ x,
-                             T* __restrict__ y) {
-    __shared__ T as;
-    if (threadIdx.x == 0) {
-        const double s = *sc;
-        as = (T)(invert ? (s != 0.0 ? 1.0 / s : 0.0) : s);
-    }
-    __syncthreads();
-    const T a = as;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = a * x[i];
-}
-
 template <typename Ti, typename To>
 __global__ void k_convert(long long n, const Ti* __restrict__ x, To* __restrict__ y) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = (To)x[i];
-}
-
-// partial[blk*k + j] = sum over this block's elements of V_j . w, j in [j0, j0+CH)
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_mdot(long long n, const T* __restrict__ V, long long ld, int k,
-                                                      const T* __restrict__ w, double* __restrict__ partial) {
-    for (int j0 = 0; j0 < k; j0 += MDOT_CHUNK) {
-        T tacc[MDOT_CHUNK];
-#pragma unroll
-        for (int q = 0; q < MDOT_CHUNK; ++q) tacc[q] = T(0);
-        int nq = min(MDOT_CHUNK, k - j0);
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-             i += (long long)gridDim.x * blockDim.x) {
-            T wi = w[i];
-#pragma unroll
-            for (int q = 0; q < MDOT_CHUNK; ++q)
-                if (q < nq) tacc[q] += V[(long long)(j0 + q) * ld + i] * wi;
-        }
-        __shared__ double outv[MDOT_CHUNK];
-        block_sum_t<T, MDOT_CHUNK>(tacc, nq, outv);
-        if (threadIdx.x < nq) partial[(long long)blockIdx.x * k + j0 + threadIdx.x] = outv[threadIdx.x];
-        __syncthreads();
-    }
 }
 
 // out[j] = sum_blk partial[blk*k + j]   (grid: k blocks)
@@ -120,63 +83,6 @@ __global__ void k_finalize(const double* __restrict__ partial, int nblk, int k, 
     __shared__ double o[1];
     block_sum<1>(v, o);
     if (threadIdx.x == 0) out[j] = o[0];
-}
-
-// w -= sum_j h_j V_j ; then partial dots V_j . w (second CGS pass)
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_update_mdot(long long n, const T* __restrict__ V, long long ld,
-                                                             int k, const double* __restrict__ h,
-                                                             T* __restrict__ w, double* __restrict__ partial) {
-    __shared__ T hs[128];
-    for (int j = threadIdx.x; j < k; j += blockDim.x) hs[j] = (T)h[j];
-    __syncthreads();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        T s = T(0);
-        for (int j = 0; j < k; ++j) s += hs[j] * V[(long long)j * ld + i];
-        w[i] = w[i] - s;
-    }
-    // the elements this thread wrote are re-read by the same thread below
-    for (int j0 = 0; j0 < k; j0 += MDOT_CHUNK) {
-        T tacc[MDOT_CHUNK];
-#pragma unroll
-        for (int q = 0; q < MDOT_CHUNK; ++q) tacc[q] = T(0);
-        int nq = min(MDOT_CHUNK, k - j0);
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-             i += (long long)gridDim.x * blockDim.x) {
-            T wi = w[i];
-#pragma unroll
-            for (int q = 0; q < MDOT_CHUNK; ++q)
-                if (q < nq) tacc[q] += V[(long long)(j0 + q) * ld + i] * wi;
-        }
-        __shared__ double outv[MDOT_CHUNK];
-        block_sum_t<T, MDOT_CHUNK>(tacc, nq, outv);
-        if (threadIdx.x < nq) partial[(long long)blockIdx.x * k + j0 + threadIdx.x] = outv[threadIdx.x];
-        __syncthreads();
-    }
-}
-
-// w -= sum_j h_j V_j ; partial |w|^2
-template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_update_norm(long long n, const T* __restrict__ V, long long ld,
-                                                             int k, const double* __restrict__ h,
-                                                             T* __restrict__ w, double* __restrict__ partial) {
-    __shared__ T hs[128];
-    for (int j = threadIdx.x; j < k; j += blockDim.x) hs[j] = (T)h[j];
-    __syncthreads();
-    T acc = T(0);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        T s = T(0);
-        for (int j = 0; j < k; ++j) s += hs[j] * V[(long long)j * ld + i];
-        T wi = w[i] - s;
-        w[i] = wi;
-        acc += wi * wi;
-    }
-    T v[1] = {acc};
-    __shared__ double o[1];
-    block_sum_t<T, 1>(v, 1, o);
-    if (threadIdx.x == 0) partial[blockIdx.x] = o[0];
 }
 
 template <typename T>
@@ -238,27 +144,23 @@ __device__ __forceinline__ void add_keep(float x, float& s, float& e) {
 }
 __device__ __forceinline__ void add_keep(double x, double& s, double&) { s += x; }
 
-// blockIdx.y: component c; partial[blk*C + c]; vec: m % 4 == 0 and x aligned for 4-entry loads
+// blockIdx.y: component c; partial[blk*C + c]; m a multiple of four, x 16-byte aligned
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_block_sums_acc(long long m, int C, const T* __restrict__ x,
-                                                                double* __restrict__ partial, int vec) {
+                                                                double* __restrict__ partial) {
     const int c = blockIdx.y;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const T* xc = x + (long long)c * m;
     T s0 = T(0), e0 = T(0), s1 = T(0), e1 = T(0);
-    if (vec) {
-        struct alignas(16) P4 {
-            T v[4];
-        };
-        for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < m / 4; q += stride) {
-            const P4 a = reinterpret_cast<const P4*>(xc)[q];
-            add_keep(a.v[0], s0, e0);
-            add_keep(a.v[1], s1, e1);
-            add_keep(a.v[2], s0, e0);
-            add_keep(a.v[3], s1, e1);
-        }
-    } else {
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += stride) add_keep(xc[i], s0, e0);
+    struct alignas(16) P4 {
+        T v[4];
+    };
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < m / 4; q += stride) {
+        const P4 a = reinterpret_cast<const P4*>(xc)[q];
+        add_keep(a.v[0], s0, e0);
+        add_keep(a.v[1], s1, e1);
+        add_keep(a.v[2], s0, e0);
+        add_keep(a.v[3], s1, e1);
     }
     double v[1] = {((double)s0 + (double)s1) + ((double)e0 + (double)e1)};
     __shared__ double o[1];
@@ -284,7 +186,7 @@ __global__ void k_subtract_means(long long m, T* __restrict__ x, const double* _
 __global__ void k_arnoldi_column(double* H, int ldh, const double* h1, const double* h2, const double* nrm2, int j,
                                  double* cs, double* sn, double* gv, double* res_out, double* inv_norm_out) {
     double* col = H + (long long)j * ldh;
-    for (int i = 0; i <= j; ++i) col[i] = h1[i] + (h2 ? h2[i] : 0.0);
+    for (int i = 0; i <= j; ++i) col[i] = h1[i] + h2[i];
     double nr = sqrt(fmax(*nrm2, 0.0));
     col[j + 1] = nr;
     *inv_norm_out = nr > 0.0 ? 1.0 / nr : 0.0;
@@ -973,12 +875,12 @@ __global__ void k_df_scale(long long n, const double* __restrict__ inv_norm, con
 // Swirydowicz, Langou, Ananthan, Yang, Thomas, "Low synchronization Gram-Schmidt
 // and generalized minimal residual algorithms", 2021).  L is formed where a vector
 // is made: the last pass, which has the block in registers, also forms its dots
-// with the remainder.  Two FP64 FMAs per entry and vector, as with one vector per
-// pass, but w moves once per block: 18 bytes per entry and vector instead of 32.
-// The FP64 pipe bounds it (89 % busy; 128^3: 28.5 us per vector, 48 with one vector
-// per pass, whose loads and sums did not overlap; whole solves at 128^3 61.3 ->
-// 52.9 ms, 192^3 299 -> 254 ms, and 512^2 53.0 -> 41.8 ms against CGS2).  A pass leaves one partial sum
-// per block of threads and dot; the next pass sums them itself, in every block and
+// with the remainder.  k vectors take 2 k + 1 FP64 FMAs per entry, as with one vector
+// per pass, and k mod 8 more for L; but w moves once per block: 18 bytes per entry and
+// vector instead of 32.  The FP64 pipe bounds it (93-95 % busy; 128^3: 28.5 us per vector, 48
+// with one vector per pass, whose loads and sums did not overlap; whole solves at
+// 128^3 61.3 -> 52.9 ms, 192^3 299 -> 254 ms, and 512^2 53.0 -> 41.8 ms against CGS2).
+// A pass leaves one partial sum per block of threads and dot; the next pass sums them itself, in every block and
 // in a fixed order (bitwise the same value everywhere), and block 0 records the
 // coefficients.
 constexpr int MGS_B = 8;
@@ -1451,33 +1353,26 @@ __global__ void k_subtract_means_v(long long m, T* __restrict__ x, const double*
 }
 
 // ---- the vector passes of the inner solve (up to INNER_MAX directions) --------
+// (four entries per 16-byte access: every axis has an even number of cells, so a field
+// is a multiple of four, and the vectors are allocations of their own)
 template <int K, typename T>
 __global__ void __launch_bounds__(256) k_inner_direction(long long n, T* __restrict__ w, const T* __restrict__ r,
                                                          const T* __restrict__ V, long long ld,
-                                                         const double* __restrict__ y, int vec) {
+                                                         const double* __restrict__ y) {
     pdl_start(w, r, V, y);
     T c[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) c[i] = (T)y[i];
     const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (vec) {
-        for (long long q = t0; q < n / 4; q += stride) {
-            Q4<T> a = reinterpret_cast<const Q4<T>*>(w)[q];
+    for (long long q = t0; q < n / 4; q += stride) {
+        Q4<T> a = reinterpret_cast<const Q4<T>*>(w)[q];
 #pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const Q4<T> v = reinterpret_cast<const Q4<T>*>(i == 0 ? r : V + (i - 1) * ld)[q];
+        for (int i = 0; i < K; ++i) {
+            const Q4<T> v = reinterpret_cast<const Q4<T>*>(i == 0 ? r : V + (i - 1) * ld)[q];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) a.v[e] -= c[i] * v.v[e];
-            }
-            reinterpret_cast<Q4<T>*>(w)[q] = a;
+            for (int e = 0; e < 4; ++e) a.v[e] -= c[i] * v.v[e];
         }
-    } else {
-        for (long long q = t0; q < n; q += stride) {
-            T a = w[q];
-#pragma unroll
-            for (int i = 0; i < K; ++i) a -= c[i] * (i == 0 ? r : V + (i - 1) * ld)[q];
-            w[q] = a;
-        }
+        reinterpret_cast<Q4<T>*>(w)[q] = a;
     }
 }
 
@@ -1486,7 +1381,7 @@ template <int K, typename T>
 __global__ void __launch_bounds__(256) k_inner_combine(long long m, const T* __restrict__ Z, long long ld,
                                                        const double* __restrict__ y, T* __restrict__ x, int d,
                                                        double* __restrict__ means, double* __restrict__ partial,
-                                                       unsigned* __restrict__ ticket, int vec) {
+                                                       unsigned* __restrict__ ticket) {
     pdl_start(Z, y);
     T c[K];
 #pragma unroll
@@ -1497,32 +1392,22 @@ __global__ void __launch_bounds__(256) k_inner_combine(long long m, const T* __r
     const long long stride = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     T s0 = T(0), e0 = T(0), s1 = T(0), e1 = T(0);
     const bool sum = means != nullptr && cmp < d;
-    if (vec) {
-        for (long long q = t0; q < m / 4; q += stride) {
-            Q4<T> a;
+    for (long long q = t0; q < m / 4; q += stride) {
+        Q4<T> a;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) a.v[e] = T(0);
+        for (int e = 0; e < 4; ++e) a.v[e] = T(0);
 #pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const Q4<T> v = reinterpret_cast<const Q4<T>*>(Z + i * ld)[q];
+        for (int i = 0; i < K; ++i) {
+            const Q4<T> v = reinterpret_cast<const Q4<T>*>(Z + i * ld)[q];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) a.v[e] += c[i] * v.v[e];
-            }
-            reinterpret_cast<Q4<T>*>(x)[q] = a;
-            if (sum) {
-                add_keep(a.v[0], s0, e0);
-                add_keep(a.v[1], s1, e1);
-                add_keep(a.v[2], s0, e0);
-                add_keep(a.v[3], s1, e1);
-            }
+            for (int e = 0; e < 4; ++e) a.v[e] += c[i] * v.v[e];
         }
-    } else {
-        for (long long q = t0; q < m; q += stride) {
-            T a = T(0);
-#pragma unroll
-            for (int i = 0; i < K; ++i) a += c[i] * Z[i * ld + q];
-            x[q] = a;
-            if (sum) add_keep(a, s0, e0);
+        reinterpret_cast<Q4<T>*>(x)[q] = a;
+        if (sum) {
+            add_keep(a.v[0], s0, e0);
+            add_keep(a.v[1], s1, e1);
+            add_keep(a.v[2], s0, e0);
+            add_keep(a.v[3], s1, e1);
         }
     }
     if (!sum) return;
@@ -1758,12 +1643,6 @@ void vec_axpby(long long n, double a, const T* x, double b, T* y, cudaStream_t s
     k_axpby<T><<<blocks_for(n), 256, 0, s>>>(n, (T)a, x, (T)b, y);
     IBR_CHECK_LAUNCH();
 }
-template <typename T>
-void vec_scale_copy(long long n, const double* scale_dev, bool invert, const T* x, T* y, cudaStream_t s) {
-    ProfScope ps(KID_SCALE, s, 2.0 * n * sizeof(T));
-    k_scale_copy<T><<<blocks_for(n), 256, 0, s>>>(n, scale_dev, invert ? 1 : 0, x, y);
-    IBR_CHECK_LAUNCH();
-}
 template <typename Ti, typename To>
 void vec_convert(long long n, const Ti* x, To* y, cudaStream_t s) {
     ProfScope ps(KID_CONVERT, s, (double)n * (sizeof(Ti) + sizeof(To)));
@@ -1771,32 +1650,6 @@ void vec_convert(long long n, const Ti* x, To* y, cudaStream_t s) {
         k_convert_v<Ti, To><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, x, y);
     else
         k_convert<Ti, To><<<blocks_for(n), 256, 0, s>>>(n, x, y);
-    IBR_CHECK_LAUNCH();
-}
-template <typename T>
-void mdot(long long n, const T* V, long long ld, int k, const T* w, double* partial, double* out, cudaStream_t s) {
-    ProfScope ps(KID_MDOT, s, (k + 1.0) * n * sizeof(T));
-    k_mdot<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, V, ld, k, w, partial);
-    IBR_CHECK_LAUNCH();
-    k_finalize<<<k, RED_THREADS, 0, s>>>(partial, RED_BLOCKS, k, out);
-    IBR_CHECK_LAUNCH();
-}
-template <typename T>
-void update_mdot(long long n, const T* V, long long ld, int k, const double* h, T* w, double* partial, double* out,
-                 cudaStream_t s) {
-    ProfScope ps(KID_UPD_MDOT, s, (k + 2.0) * n * sizeof(T));
-    k_update_mdot<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, V, ld, k, h, w, partial);
-    IBR_CHECK_LAUNCH();
-    k_finalize<<<k, RED_THREADS, 0, s>>>(partial, RED_BLOCKS, k, out);
-    IBR_CHECK_LAUNCH();
-}
-template <typename T>
-void update_norm2(long long n, const T* V, long long ld, int k, const double* h, T* w, double* partial, double* out,
-                  cudaStream_t s) {
-    ProfScope ps(KID_UPD_NORM, s, (k + 2.0) * n * sizeof(T));
-    k_update_norm<T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, V, ld, k, h, w, partial);
-    IBR_CHECK_LAUNCH();
-    k_finalize<<<1, RED_THREADS, 0, s>>>(partial, RED_BLOCKS, 1, out);
     IBR_CHECK_LAUNCH();
 }
 template <typename T>
@@ -1826,9 +1679,10 @@ void combine(long long n, const Tz* Z, long long ld, int k, const double* y, T* 
 template <typename T>
 void inner_direction(long long n, T* w, const T* r, const T* V, long long ld, int k, const double* y, cudaStream_t s) {
     ProfScope ps(KID_UPD_NORM, s, (k + 2.0) * n * sizeof(T));
-    const int vec = n % 4 == 0 && vec16(r) && vec16(w) && vec16_basis(V, ld) ? 1 : 0;
-    const dim3 grid((unsigned)std::min<long long>(8 * 152, n / (vec ? 1024 : 256) + 1));
-    auto go = [&](auto* kern) { launch_k(kern, grid, dim3(256), 0, s, n, w, r, V, ld, y, vec); };
+    if (n % 4 != 0 || !vec16(r) || !vec16(w) || !vec16_basis(V, ld))
+        throw Error{IBR_EINVAL, "inner_direction: a multiple of four entries, 16-byte aligned"};
+    const dim3 grid((unsigned)std::min<long long>(8 * 152, n / 1024 + 1));
+    auto go = [&](auto* kern) { launch_k(kern, grid, dim3(256), 0, s, n, w, r, V, ld, y); };
     if (k == 1) go(k_inner_direction<1, T>);
     else if (k == 2) go(k_inner_direction<2, T>);
     else if (k == 3) go(k_inner_direction<3, T>);
@@ -1839,9 +1693,10 @@ template <typename T>
 void inner_combine(long long m, int nc, const T* Z, long long ld, int k, const double* y, T* x, int d, double* means,
                    double* partial, unsigned* ticket, cudaStream_t s) {
     ProfScope ps(KID_COMBINE, s, (k + 1.0) * m * nc * sizeof(T));
-    const int vec = m % 4 == 0 && vec16(x) && vec16_basis(Z, ld) ? 1 : 0;
-    const dim3 grid((unsigned)std::min<long long>(152, m / (vec ? 1024 : 256) + 1), (unsigned)nc);
-    auto go = [&](auto* kern) { launch_k(kern, grid, dim3(256), 0, s, m, Z, ld, y, x, d, means, partial, ticket, vec); };
+    if (m % 4 != 0 || !vec16(x) || !vec16_basis(Z, ld))
+        throw Error{IBR_EINVAL, "inner_combine: blocks of a multiple of four entries, 16-byte aligned"};
+    const dim3 grid((unsigned)std::min<long long>(152, m / 1024 + 1), (unsigned)nc);
+    auto go = [&](auto* kern) { launch_k(kern, grid, dim3(256), 0, s, m, Z, ld, y, x, d, means, partial, ticket); };
     if (k == 1) go(k_inner_combine<1, T>);
     else if (k == 2) go(k_inner_combine<2, T>);
     else if (k == 3) go(k_inner_combine<3, T>);
@@ -1866,7 +1721,9 @@ template <typename T>
 void block_means_acc(long long m, int C, const T* x, double* partial, double* out, cudaStream_t s) {
     ProfScope ps(KID_BLOCK_MEANS, s, (double)m * C * sizeof(T));
     const int blocks = (int)std::min<long long>(RED_BLOCKS / 4, (m / 4 + RED_THREADS - 1) / RED_THREADS + 1);
-    k_block_sums_acc<T><<<dim3(blocks, C), RED_THREADS, 0, s>>>(m, C, x, partial, m % 4 == 0 && vec16(x) ? 1 : 0);
+    if (m % 4 != 0 || !vec16(x))
+        throw Error{IBR_EINVAL, "block_means_acc: blocks of a multiple of four entries, 16-byte aligned"};
+    k_block_sums_acc<T><<<dim3(blocks, C), RED_THREADS, 0, s>>>(m, C, x, partial);
     IBR_CHECK_LAUNCH();
     k_finalize<<<C, RED_THREADS, 0, s>>>(partial, blocks, C, out);
     IBR_CHECK_LAUNCH();
@@ -1902,12 +1759,6 @@ void hess_solve(const double* H, int ldh, const double* gv, int k, double* y, cu
 
 #define IBR_INST(T)                                                                                              \
     template void vec_axpby<T>(long long, double, const T*, double, T*, cudaStream_t);                          \
-    template void vec_scale_copy<T>(long long, const double*, bool, const T*, T*, cudaStream_t);                \
-    template void mdot<T>(long long, const T*, long long, int, const T*, double*, double*, cudaStream_t);       \
-    template void update_mdot<T>(long long, const T*, long long, int, const double*, T*, double*, double*,      \
-                                 cudaStream_t);                                                                 \
-    template void update_norm2<T>(long long, const T*, long long, int, const double*, T*, double*, double*,     \
-                                  cudaStream_t);                                                                \
     template void norm2<T>(long long, const T*, double*, double*, cudaStream_t);                                \
     template void inner_direction<T>(long long, T*, const T*, const T*, long long, int, const double*, cudaStream_t); \
     template void inner_combine<T>(long long, int, const T*, long long, int, const double*, T*, int, double*, double*, \

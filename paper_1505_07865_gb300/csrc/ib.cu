@@ -337,14 +337,12 @@ __device__ __forceinline__ T interp_warp(const Geo& g, int ia, const int* __rest
 
 template <int D, int KW, typename T, typename Tadd>
 __global__ void k_interp(Geo g, int N, const int* __restrict__ idx, const T* __restrict__ w, const T* __restrict__ v,
-                         T* __restrict__ out, T sign, const Tadd* __restrict__ add, T add_scale,
-                         const double* __restrict__ mean) {
+                         T* __restrict__ out, T sign, const Tadd* __restrict__ add, T add_scale) {
     const int ia = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (ia >= N * D) return;
     const T acc = interp_warp<D, KW, T>(g, ia, idx, w, v);
     if ((threadIdx.x & 31) == 0) {
-        // the weights of a window sum to one: J (v - m) = J v - m
-        T r = sign * (mean ? acc - (T)mean[ia % D] : acc);
+        T r = sign * acc;
         if (add) r += add_scale * (T)add[ia];
         out[ia] = r;
     }
@@ -373,6 +371,7 @@ __global__ void __launch_bounds__(128) k_spread_interp(Geo g, int N, int nsb, lo
     const int ia = (((int)blockIdx.x - nsb) * (int)blockDim.x + (int)threadIdx.x) >> 5;
     if (ia >= N * D) return;
     const double acc = interp_warp<D, KW, double>(g, ia, idx, w, v);
+    // the weights of a window sum to one: J (v - mean) = J v - mean
     if ((threadIdx.x & 31) == 0) out[ia] = sign * (mean ? acc - mean[ia % D] : acc);
 }
 
@@ -575,7 +574,7 @@ void spread_gather(const MarkerData& md, const T* lam, T* y, double scale, cudaS
 
 template <typename T, typename Tadd>
 void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign, const Tadd* add, cudaStream_t s,
-            double add_scale, const double* mean) {
+            double add_scale) {
     const T* w = sizeof(T) == 8 ? reinterpret_cast<const T*>(md.w64) : reinterpret_cast<const T*>(md.w32);
     int threads = 128;
     int blocks = grid_1d((long long)md.N * g.d * 32, threads);
@@ -584,18 +583,14 @@ void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign,
                  (double)md.N * g.d * ((g.d == 3 ? kw * kw * kw : kw * kw) * sizeof(T) + g.d * kw * sizeof(T) + sizeof(T)));
     if (g.d == 3) {
         if (kw == 6)
-            k_interp<3, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
-                                                          mean);
+            k_interp<3, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
         else
-            k_interp<3, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
-                                                          mean);
+            k_interp<3, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
     } else {
         if (kw == 6)
-            k_interp<2, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
-                                                          mean);
+            k_interp<2, 6, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
         else
-            k_interp<2, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale,
-                                                          mean);
+            k_interp<2, 4, T, Tadd><<<blocks, threads, 0, s>>>(g, md.N, md.idx, w, v, out, (T)sign, add, (T)add_scale);
     }
     IBR_CHECK_LAUNCH();
 }
@@ -647,9 +642,9 @@ void rigid_KT(int d, int B, const int* body_start, const double* rel, const doub
 template void spread_gather<double>(const MarkerData&, const double*, double*, double, cudaStream_t);
 template void spread_gather<float>(const MarkerData&, const float*, float*, double, cudaStream_t);
 template void interp<double, double>(const Geo&, const MarkerData&, const double*, double*, double, const double*,
-                                     cudaStream_t, double, const double*);
+                                     cudaStream_t, double);
 template void interp<float, double>(const Geo&, const MarkerData&, const float*, float*, double, const double*,
-                                    cudaStream_t, double, const double*);
+                                    cudaStream_t, double);
 template void lam_sum<double>(int, int, const double*, double, double*, cudaStream_t);
 template void lam_sum<float>(int, int, const float*, double, double*, cudaStream_t);
 

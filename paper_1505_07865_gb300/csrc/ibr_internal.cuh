@@ -390,23 +390,8 @@ constexpr int RED_THREADS = 256;
 constexpr int MDOT_CHUNK = 8;
 template <typename T>
 void vec_axpby(long long n, double a, const T* x, double b, T* y, cudaStream_t s);   // y = a x + b y
-template <typename T>
-void vec_scale_copy(long long n, const double* scale_dev, bool invert, const T* x, T* y,
-                    cudaStream_t s);  // y = x * (invert ? 1/scale : scale)
 template <typename Ti, typename To>
 void vec_convert(long long n, const Ti* x, To* y, cudaStream_t s);
-// partial dots of w against k vectors V + j*ld, summed into out[0..k) (double)
-template <typename T>
-void mdot(long long n, const T* V, long long ld, int k, const T* w, double* partial, double* out,
-          cudaStream_t s);
-// w -= sum_j h[j] V_j, then out[j] = V_j . w (CGS2 second pass); h device
-template <typename T>
-void update_mdot(long long n, const T* V, long long ld, int k, const double* h, T* w, double* partial,
-                 double* out, cudaStream_t s);
-// w -= sum_j h[j] V_j, then out[0] = w . w
-template <typename T>
-void update_norm2(long long n, const T* V, long long ld, int k, const double* h, T* w, double* partial,
-                  double* out, cudaStream_t s);
 template <typename T>
 void norm2(long long n, const T* w, double* partial, double* out, cudaStream_t s);
 // x (+)= sum_j y[j] Z_j  (y device)
@@ -462,8 +447,8 @@ struct __align__(8) dflt {
 // of its first n32 entries (out32, may be NULL) and an FP64 one of the entries
 // from64 .. n64 - 1 (out64): h[0..k) the coefficients, st[2] = |w_perp|^2, st[3] its
 // inverse square root, st[1] = 0; column k - 1 of
-// H with its Givens rotation as arnoldi_column does it.  Eight vectors per pass
-// and two FP64 FMAs per entry and vector; w is overwritten.  n and ld even
+// H with its Givens rotation as arnoldi_column does it.  Eight vectors per pass,
+// 2 k + 1 + (k mod 8) FP64 FMAs per entry; w is overwritten.  n and ld even
 // (entries past the system length are a zero pad of w and of every basis vector),
 // V, w, vout, out32 16-byte aligned, 1 <= k <= 127; partial holds 2 * 9 * 304
 // doubles, gram 8 (k + 1): the dots of the basis vectors of one block of eight,
@@ -530,11 +515,10 @@ void markers_build_gather(const Geo& g, MarkerData& md, cudaStream_t s);
 // y[face] += scale * sum w * lam   (no atomics; one thread per touched face)
 template <typename T>
 void spread_gather(const MarkerData& md, const T* lam, T* y, double scale, cudaStream_t s);
-// out[i*d+a] = sign * (J (v - mean))_i^a + (add ? add_scale * add[i*d+a] : 0);
-// mean: d doubles on the device or NULL (zero)
+// out[i*d+a] = sign * (J v)_i^a + (add ? add_scale * add[i*d+a] : 0)
 template <typename T, typename Tadd>
 void interp(const Geo& g, const MarkerData& md, const T* v, T* out, double sign, const Tadd* add,
-            cudaStream_t s, double add_scale, const double* mean = nullptr);
+            cudaStream_t s, double add_scale);
 // The marker part of a product with the system matrix in one launch: y (fluid
 // rows) += scale S lam, out = sign J (v - mean) as spread_gather and interp do them
 void spread_interp(const Geo& g, const MarkerData& md, const double* lam, double* y, double scale, const double* v,

@@ -466,7 +466,6 @@ struct PC {
         combine<T, T>(nS, Zi, nS, ns, yv, xout, false, s);
     }
 
-    // z = P^-1 r for the constrained system (Sec. V.A), FP64 in and out
     // steps 1-4 of Sec. V.A from rs (fluid part, precision T) and rL (the
     // constraint part, FP64) into xs (v, pi) and lamT (Lambda); fixed buffers
     // only, so the whole sequence can be captured as one CUDA graph
@@ -504,7 +503,7 @@ struct PC {
         // constrained problem.  Uniform fields lie in the null space of the fluid
         // rows, so the vector itself is left as it is and only the mean velocity
         // is measured: the product with the matrix takes it out of the
-        // constraint rows (full_matvec), and the solution is projected at the
+        // constraint rows (marker_rows), and the solution is projected at the
         // end of each cycle.  Subtracting it from the entries in the
         // preconditioner's precision left a mean of about 1e-9 |v| after
         // rounding, which the final projection turned into an error of the
@@ -1281,7 +1280,7 @@ void project_solution(ibr_grid* G, double* x) {
 
 // The outer Arnoldi orthogonalisation, over the FP64 basis in both
 // precisions: modified Gram-Schmidt, eight vectors per pass (blas.cu).  On this
-// part the FP64 pipe bounds it, with two FMAs per entry and basis vector;
+// part the FP64 pipe bounds it, with little more than two FMAs per entry and vector;
 // classical Gram-Schmidt with reorthogonalisation (CGS2) needs four, and its eight
 // launches per step are no gain on small systems either, where the blocked form has
 // k / 8 + 2 (solves at 64^3 34.1 -> 27.1 ms, 256^2 13.7 -> 12.6, 64^2 6.0 -> 5.6).
@@ -1306,8 +1305,10 @@ int arnoldi_kind() {
 // on with the basis it has and a stricter estimate (the iterate at its start is
 // kept in xc), instead of being given up: a new cycle starts from a residual of
 // rounding noise and needs about ten steps to gain what one or two more steps of
-// the old one do.  Where going on does not help (the residual stays above three
-// quarters of what it was), the cycle ends there as it would have.
+// the old one do.  It goes on while the part of the residual that the estimate does
+// not explain, (rn^2 - est^2)^(1/2), is below the target: the next estimate to be met is
+// 0.7 of what that part leaves of it.  Where rounding alone exceeds the target, the
+// cycle ends there.
 int fgmres(ibr_grid* G, const ibr_solve_opts& o, ibr_solve_info& info, bool warm = false) {
     cudaStream_t s = G->stream;
     long long len = G->len;

@@ -208,9 +208,12 @@ __global__ void __launch_bounds__(256) k_stokes(const T* __restrict__ x, T* __re
 // significands with six more bits below; 59 bits, so a sum of twelve fits), added
 // exactly, and rounded once on conversion back.  That leaves 14 FP64 operations
 // per cell, the rest runs on the integer pipe beside them.  A value's bits below
-// 2^-6 ulp of the largest are cut off, so the sum is closer to the exact one than
-// FP64 additions, each rounded at the size of the neighbours' sum.  Exponents near
-// either end of the range, infinities and NaN take the plain formula.  Measured as
+// 2^-6 ulp of the largest are cut off: at most 12 x 2^-58 of the largest value, less
+// than the roundings of FP64 additions may add up to (each 2^-53 of a partial sum).
+// Not so for every sum: where large terms cancel exactly, FP64 additions in a lucky
+// order keep a small term that is cut off here (2^70 - 2^70 + 1 gives 0).  Exponents
+// near either end of the range, coefficients that are no normal numbers, infinities and
+// NaN take the plain formula.  Measured as
 // whole products with the system matrix (marker terms included): 128^3 169 -> 105
 // us, 160^3 348 -> 216 us, 64^3 41 -> 33 us, 512^2 27 -> 24 us.  Walls keep the
 // plain kernel (their rules change the terms of a sum from cell to cell).
@@ -2015,26 +2018,20 @@ void stokes_apply(const Geo& g, const T* x, T* y, double sigma, double eta, cons
     T kh2 = (T)(eta / (g.h * g.h));
     T ih = (T)(1.0 / g.h);
     dim3 grid((g.n0 + BX - 1) / BX, (g.n1 + BY - 1) / BY, g.n2), blk(BX, BY);
-    ProfScope ps(KID_STOKES, s, 2.0 * (g.d + 1) * g.ncell * sizeof(T));
-    const bool w = g.wall != 0;
-    if constexpr (std::is_same<T, double>::value) {
-        if (!w) {
-            stokes_apply_from<double>(g, x, y, nullptr, sigma, eta, shift_dev, s);
-            return;
-        }
-    }
-    if (g.d == 3) {
-        if (w)
-            launch_k(k_stokes<3, true, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih, shift_dev);
-        else
-            launch_k(k_stokes<3, false, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih, shift_dev);
+    const double bytes = 2.0 * (g.d + 1) * g.ncell * sizeof(T);
+    if (g.wall) {
+        ProfScope ps(KID_STOKES, s, bytes);
+        launch_k(g.d == 3 ? k_stokes<3, true, T> : k_stokes<2, true, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih,
+                 shift_dev);
+        IBR_CHECK_LAUNCH();
+    } else if constexpr (std::is_same<T, double>::value) {
+        stokes_apply_from<double>(g, x, y, nullptr, sigma, eta, shift_dev, s);
     } else {
-        if (w)
-            launch_k(k_stokes<2, true, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih, shift_dev);
-        else
-            launch_k(k_stokes<2, false, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih, shift_dev);
+        ProfScope ps(KID_STOKES, s, bytes);
+        launch_k(g.d == 3 ? k_stokes<3, false, T> : k_stokes<2, false, T>, grid, blk, 0, s, x, y, g, (T)sigma, kh2, ih,
+                 shift_dev);
+        IBR_CHECK_LAUNCH();
     }
-    IBR_CHECK_LAUNCH();
 }
 
 template <typename T>
@@ -2531,8 +2528,9 @@ void mg_vcycle(const Geo* lev, int L, T* const* U, T* const* Fw, const T* F0, in
     // The tail runs on one SM per field.  Where its larger levels can run on many
     // and that is faster, they do: FP64 sweeps, at two operations per clock and SM,
     // from 32^2 and 8^3 up (FP64 P_S on 64^2 76 us, 135 with that level in the
-    // tail; on 64^3 387, 421), and FP32 with walls, whose boundary rules cost
-    // registers, from 32^2 up (64^2 61 us, 70); FP32 on periodic grids keeps them.
+    // tail; on 64^3 387, 421; between walls on 16^3 178, 259, on 32^3 333, 424, on 64^3
+    // 634, 722), and FP32 with walls, whose boundary rules cost registers, from 32^2 up
+    // (64^2 61 us, 70); FP32 on periodic grids keeps them.
     const long long most = sizeof(T) == 8 ? (lev[0].d == 2 ? 1024 : 512)
                                           : (lev[0].d == 2 && lev[0].wall ? 1024 : MG_TAIL_MAX_CELLS);
     if (!use_cluster)

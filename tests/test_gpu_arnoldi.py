@@ -1,9 +1,8 @@
 """The outer FGMRES orthogonalisations against each other, on the same solves:
 classical Gram-Schmidt with reorthogonalisation over the FP64 basis,
-pipelined on bulk copies (IBR_ARNOLDI=cgs2; the default below two million
-entries), against modified Gram-Schmidt over the FP64 basis (=mgs; the
-default from two million entries) and CGS2 over a double-float basis (=df:
-pairs of floats, arithmetic on the FP32 pipe).
+pipelined on bulk copies (IBR_ARNOLDI=cgs2), against modified Gram-Schmidt
+over the FP64 basis (=mgs, the default: eight vectors per pass) and CGS2 over a
+double-float basis (=df: pairs of floats, arithmetic on the FP32 pipe).
 
 Every run must converge to the solve tolerance and agree with the oracle's
 exact solution (and with the CGS2 run) to the accuracy that tolerance

@@ -2,8 +2,9 @@
 one launch each and the one-block tail, at sizes where tiles, halos and pairs of
 cells do not fit evenly, for both precisions.
 
-Reference: ibr_op_vcycle_noalloc, which has no temporaries for the legs and runs
-the per-level kernels (FP64).  The kernels apply the same
+Reference: ibr_op_vcycle_noalloc (FP64), which has no temporaries for the legs: it runs
+the per-level kernels down to the one-block tail, and the tail itself on levels of at
+most 4096 cells (test_gpu_mg_reference.py pins that one independently).  The kernels apply the same
 formulas in the same order up to the association of two sums, so FP64 agrees to
 1e-13 of the largest value after two cycles of a contraction; FP32 rounding of
 about 30 operations per cell and level gives 1e-5.
