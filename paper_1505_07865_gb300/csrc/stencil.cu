@@ -213,9 +213,9 @@ __global__ void __launch_bounds__(256) k_stokes(const T* __restrict__ x, T* __re
 // Not so for every sum: where large terms cancel exactly, FP64 additions in a lucky
 // order keep a small term that is cut off here (2^70 - 2^70 + 1 gives 0).  Exponents
 // near either end of the range, coefficients that are no normal numbers, infinities and
-// NaN take the plain formula.  Measured as
-// whole products with the system matrix (marker terms included): 128^3 169 -> 105
-// us, 160^3 348 -> 216 us, 64^3 41 -> 33 us, 512^2 27 -> 24 us.  Walls keep the
+// NaN take the plain formula.  Measured as whole products with the system matrix (marker
+// terms included): 128^3 169 -> 99 us, 160^3 348 -> 204, 64^3 41 -> 25, 512^2 27 -> 18.  The
+// FP64 pipe is still what bounds it (83 % busy, the integer pipe 45 %).  Walls keep the
 // plain kernel (their rules change the terms of a sum from cell to cell).
 __device__ __forceinline__ int fx_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 __device__ __forceinline__ long long fx_int(double v, int emax) {
